@@ -61,10 +61,10 @@ extern "C" {
 #define ESMF_PREC_FP16X2  2   /* integrals as scaled FP16 hi+lo pairs, tensor */
                               /* cores with FP32 accumulation (stored only)   */
 #define ESMF_PREC_BF16X2  3   /* as FP16X2 with BF16 halves (ablation)        */
-#define ESMF_PREC_F32X2   4   /* FP64 integrals contracted in double-FP32     */
-                              /* (hi+lo) arithmetic on CUDA cores: error-free */
-                              /* products (FMA) and compensated sums (TwoSum),*/
-                              /* about 2^-44 relative, at FP32-pipe rates;    */
+#define ESMF_PREC_F32X2   4   /* FP64 integrals kept as FP32 hi+lo pairs; on  */
+                              /* the CUDA-core path contracted in double-FP32 */
+                              /* (error-free products by FMA, compensated     */
+                              /* sums by TwoSum): about 2^-44 relative;       */
                               /* stored only                                   */
 
 /*
@@ -369,10 +369,12 @@ int esmf_fock_build_host(esmf_fock_t *h, int m, const double *D_host,
 int esmf_fock_set_density_screening(esmf_fock_t *h, double tol_d);
 
 /*
- * Contraction kernel choice for split 16-bit stores (FP16X2 / BF16X2):
- * ESMF_PATH_AUTO uses the tensor-core kernel, ESMF_PATH_CUDA_CORE the
- * CUDA-core kernel (same results within rounding; kept as a cross-check).
- * Other precisions always use the CUDA-core kernels.  Errors: INVALID_ARG.
+ * Contraction kernel choice for stored FP64, F32X2, FP16X2 and BF16X2
+ * integrals: ESMF_PATH_AUTO uses the tensor-core kernels (for FP64 and F32X2
+ * by error-free splitting, as accurate as FP64 arithmetic),
+ * ESMF_PATH_CUDA_CORE the CUDA-core kernels (same results within rounding;
+ * kept as a cross-check).  FP32 stores and integral-direct FP64 / FP32
+ * handles always use the CUDA-core kernels.  Errors: INVALID_ARG.
  */
 #define ESMF_PATH_AUTO       0
 #define ESMF_PATH_CUDA_CORE  1

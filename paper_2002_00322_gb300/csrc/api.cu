@@ -108,8 +108,15 @@ struct esmf_fock {
     unsigned *sched = nullptr;     // the tensor kernel's work counter
     int *err_host = nullptr, *err_dev = nullptr;   // mapped page-locked flag
     int64_t n_stored = 0, store_bytes = 0, n_kept_unique = 0;
-    // work (device)
-    double *Jacc = nullptr, *Kacc = nullptr;
+    // work (device): the FP64 accumulators of a build of m <= work_m densities,
+    // J then K (then, on the split path, K's transposed blocks and a flag word)
+    double *acc = nullptr;
+    size_t acc_n = 0;
+    // FP64 and double-FP32 stores: density digit tiles of the tensor-core path;
+    // no_split: this handle stays on the CUDA-core kernel (values beyond FP64's
+    // range, or no memory for the tiles)
+    void *skbank = nullptr, *sjbank = nullptr;
+    bool no_split = false;
     void *Dt = nullptr;            // D in the CUDA-core arithmetic type (FP32 / double-FP32), work_m densities
     double *ework = nullptr;       // ESMF energy / gradient work memory
     size_t ework_n = 0;
@@ -264,7 +271,7 @@ void release(esmf_fock *h) {
     cudaFree(h->ptab); cudaFree(h->pslot); cudaFree(h->pblocks);
     cudaFree(h->kbank); cudaFree(h->jbank); cudaFree(h->dmax); cudaFree(h->sched);
     if (h->err_host) cudaFreeHost(h->err_host);
-    cudaFree(h->Jacc); cudaFree(h->Kacc); cudaFree(h->ework); cudaFree(h->Dt);
+    cudaFree(h->acc); cudaFree(h->skbank); cudaFree(h->sjbank); cudaFree(h->ework); cudaFree(h->Dt);
     cudaFree(h->dw); cudaFree(h->dwb);
     cudaFree(h->dfB); cudaFree(h->dfB2); cudaFree(h->dfDt); cudaFree(h->dfJt); cudaFree(h->dfKt);
     cudaFree(h->dfg); cudaFree(h->dfY);
@@ -301,7 +308,28 @@ bool is_device_ptr(const void *p) {
 // chunk and contract them on the tensor cores
 bool tensor_direct(const esmf_fock *h) { return h->mode == ESMF_MODE_DIRECT && is_split16(h->prec) && h->scratch; }
 
+// FP64 or double-FP32 store that builds by exact digit splitting on the tensor
+// cores (jk_split.cu)
+bool split_path(const esmf_fock *h) {
+    return h->mode == ESMF_MODE_STORED && (h->prec == ESMF_PREC_FP64 || h->prec == ESMF_PREC_F32X2) && !h->no_split;
+}
+
+// doubles of the accumulators of a build of m densities
+size_t acc_doubles(const esmf_fock *h, int m) {
+    const size_t cnt = (size_t)m * h->np * h->np;
+    return split_path(h) ? 3 * cnt + 1 : 2 * cnt;
+}
+
 int ensure_work(esmf_fock *h, int m) {
+    if (split_path(h) && !h->skbank) {
+        // without room for the digit tiles the handle keeps the CUDA-core kernel
+        if (dalloc(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb)) != ESMF_OK ||
+            dalloc(h, (unsigned char **)&h->sjbank, split_jbank_bytes(h->nb)) != ESMF_OK) {
+            cudaGetLastError();
+            dfree(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb));
+            h->no_split = true;
+        }
+    }
     if ((h->mode == ESMF_MODE_STORED || tensor_direct(h)) && is_split16(h->prec) && !h->kbank) {
         RET(dalloc(h, (unsigned char **)&h->kbank, umma_kbank_bytes(h->nb)));
         RET(dalloc(h, (unsigned char **)&h->jbank, umma_jbank_bytes(h->nb)));
@@ -313,14 +341,17 @@ int ensure_work(esmf_fock *h, int m) {
         RET(dalloc(h, &h->dwb, (size_t)h->nb * h->nb));
     }
     if (m <= h->work_m) return ESMF_OK;
-    const size_t cnt = (size_t)m * h->np * h->np;
     const size_t tb = density_typed_bytes(h->prec);
-    dfree(h, &h->Jacc, (size_t)h->work_m * h->np * h->np);
-    dfree(h, &h->Kacc, (size_t)h->work_m * h->np * h->np);
+    dfree(h, &h->acc, h->acc_n);
     dfree(h, (unsigned char **)&h->Dt, (size_t)h->work_m * h->n * h->n * tb);
     h->work_m = 0;
-    RET(dalloc(h, &h->Jacc, cnt));
-    RET(dalloc(h, &h->Kacc, cnt));
+    h->acc_n = 0;
+    if (split_path(h) && dalloc(h, &h->acc, acc_doubles(h, m)) != ESMF_OK) {
+        cudaGetLastError();
+        h->no_split = true;
+    }
+    if (!h->acc) RET(dalloc(h, &h->acc, acc_doubles(h, m)));
+    h->acc_n = acc_doubles(h, m);
     if (tb) RET(dalloc(h, (unsigned char **)&h->Dt, (size_t)m * h->n * h->n * tb));
     h->work_m = m;
     return ESMF_OK;
@@ -671,6 +702,12 @@ static int create_impl(const esmf_basis_t *basis, const int32_t *cart, double to
         int e = 0;
         if (qmax > 0.0) std::frexp(qmax * qmax, &e);
         h->vscale = qmax > 0.0 ? (float)std::ldexp(1.0, 14 - e) : 1.0f;
+    }
+    // integrals are bounded by max Q^2: the split path takes them up to 2^500
+    {
+        double qmax = 0.0;
+        for (double x : hQ) qmax = std::isfinite(x) ? std::max(qmax, x) : x;
+        h->no_split = !(qmax <= 0x1p250);
     }
     if (!ck(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, device), "SM count"))
         return fail(ESMF_ERR_CUDA);
@@ -1222,16 +1259,16 @@ int build_range(esmf_fock_t *h, int64_t b0, int64_t b1, int m, const double *D, 
     }
     RET(ensure_work(h, m));
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t acc = sizeof(double) * (size_t)m * h->np * h->np;
-    CKR(cudaMemsetAsync(h->Jacc, 0, acc, s));
-    CKR(cudaMemsetAsync(h->Kacc, 0, acc, s));
+    const size_t cnt = (size_t)m * h->np * h->np;
+    double *const Jacc = h->acc, *const Kacc = h->acc + cnt;
+    CKR(cudaMemsetAsync(h->acc, 0, sizeof(double) * acc_doubles(h, m), s));
     if (traces) CKR(cudaMemsetAsync(traces, 0, sizeof(double) * m, s));
     if (b1 > b0) {
         JKArgs a;
         a.b = h->dev(); a.Q = h->S; a.tol = h->tol_s; a.bricks = h->bricks + b0; a.nbricks = b1 - b0;
         a.offsets = h->offsets ? h->offsets + b0 : nullptr; a.store = h->store; a.precision = h->prec;
         a.mode = h->mode;
-        a.m = m; a.D = D; a.Jacc = h->Jacc; a.Kacc = h->Kacc;
+        a.m = m; a.D = D; a.Jacc = Jacc; a.Kacc = Kacc;
         a.ptab = h->ptab; a.pslot = h->pslot;
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (h->timing && h->ev_used < 65536) {
@@ -1263,7 +1300,7 @@ int build_range(esmf_fock_t *h, int64_t b0, int64_t b1, int m, const double *D, 
             L.kbank = h->kbank; L.jbank = h->jbank;
             L.dmax_bits = h->dmax; L.D = D; L.n = h->n; L.np = h->np; L.nb = h->nb; L.m = m;
             L.bf16 = h->prec == ESMF_PREC_BF16X2; L.num_sms = h->num_sms; L.vscale = h->vscale;
-            L.Jacc = h->Jacc; L.Kacc = h->Kacc; L.error = h->err_dev; L.counter = h->sched;
+            L.Jacc = Jacc; L.Kacc = Kacc; L.error = h->err_dev; L.counter = h->sched;
             L.chunk = chunk ? chunk : 16;
             // chunks of bricks [r0, r1) for the tensor kernel: the whole list's, or
             // the range's own cost-balanced ones (scratch chunks and shards), built once
@@ -1310,7 +1347,19 @@ int build_range(esmf_fock_t *h, int64_t b0, int64_t b1, int m, const double *D, 
                 }
                 if (e1) CKR(cudaEventRecord(e1, s));
             }
-            return launch_finalize_blocked(h->dev(), m, D, h->Jacc, h->Kacc, J, K, F, traces, s);
+            return launch_finalize_blocked(h->dev(), m, D, Jacc, Kacc, nullptr, J, K, F, traces, s);
+        }
+        if (split_path(h) && h->path != ESMF_PATH_CUDA_CORE && h->tol_d == 0.0) {
+            SplitLaunch L;
+            L.bricks = a.bricks; L.nbricks = a.nbricks; L.offsets = a.offsets; L.store = h->store;
+            L.f32x2 = h->prec == ESMF_PREC_F32X2;
+            L.kbank = h->skbank; L.jbank = h->sjbank; L.D = D; L.n = h->n; L.nb = h->nb; L.m = m;
+            L.num_sms = h->num_sms;
+            L.Jacc = Jacc; L.Kacc = Kacc; L.KTacc = Kacc + cnt;
+            L.nonfinite = (int *)(Kacc + 2 * cnt); L.error = h->err_dev;
+            L.ev_start = e0; L.ev_stop = e1;
+            RET(launch_jk_split(L, s));
+            return launch_finalize_blocked(h->dev(), m, D, Jacc, Kacc, L.KTacc, J, K, F, traces, s);
         }
         if (h->Dt) {
             RET(launch_density_typed(h->prec, (int64_t)m * h->n * h->n, D, h->Dt, s));
@@ -1321,7 +1370,7 @@ int build_range(esmf_fock_t *h, int64_t b0, int64_t b1, int m, const double *D, 
         else RET(launch_jk_cuda(a, s));
         if (e1) CKR(cudaEventRecord(e1, s));
     }
-    RET(launch_finalize(h->dev(), m, D, h->Jacc, h->Kacc, J, K, F, traces, s));
+    RET(launch_finalize(h->dev(), m, D, Jacc, Kacc, J, K, F, traces, s));
     return ESMF_OK;
 }
 
@@ -1372,23 +1421,21 @@ int esmf_fock_build_batch(int count, esmf_fock_t *const *hs, const int *ms, cons
             return ESMF_ERR_INVALID_ARG;
         }
         RET(ensure_work(h, m));
-        const size_t acc = sizeof(double) * (size_t)m * h->np * h->np;
-        CKR(cudaMemsetAsync(h->Jacc, 0, acc, s));
-        CKR(cudaMemsetAsync(h->Kacc, 0, acc, s));
+        CKR(cudaMemsetAsync(h->acc, 0, sizeof(double) * acc_doubles(h, m), s));
         if (tr) CKR(cudaMemsetAsync(tr, 0, sizeof(double) * m, s));
         UmmaLaunch &l = L[i];
         l.bricks = h->bricks; l.nbricks = h->nbricks; l.offsets = h->offsets;
         l.store = (const uint32_t *)h->store; l.kbank = h->kbank; l.jbank = h->jbank;
         l.dmax_bits = h->dmax; l.D = Ds[i]; l.n = h->n; l.np = h->np; l.nb = h->nb; l.m = m;
         l.bf16 = h->prec == ESMF_PREC_BF16X2; l.num_sms = h->num_sms; l.vscale = h->vscale;
-        l.Jacc = h->Jacc; l.Kacc = h->Kacc; l.error = h->err_dev; l.counter = h->sched;
+        l.Jacc = h->acc; l.Kacc = h->acc + (size_t)m * h->np * h->np; l.error = h->err_dev; l.counter = h->sched;
         l.chunk = 16;
         if (h->parts) { l.part = h->parts; l.nparts = h->nparts; }
     }
     RET(launch_jk_umma_batch(L, count, s));
     for (int i = 0; i < count; ++i) {
         esmf_fock_t *h = hs[i];
-        RET(launch_finalize_blocked(h->dev(), ms[i], Ds[i], h->Jacc, h->Kacc, Js[i], Ks[i], Fs ? Fs[i] : nullptr,
+        RET(launch_finalize_blocked(h->dev(), ms[i], Ds[i], L[i].Jacc, L[i].Kacc, nullptr, Js[i], Ks[i], Fs ? Fs[i] : nullptr,
                                     traces ? traces[i] : nullptr, s));
     }
     return ESMF_OK;

@@ -144,14 +144,35 @@ struct UmmaLaunch {
 };
 int launch_jk_umma(const UmmaLaunch &L, cudaStream_t s);
 int launch_jk_umma_batch(const UmmaLaunch *Ls, int count, cudaStream_t s);   // count <= 16
+// KTb: further K contributions as transposed blocks ([Y][X][k][y][x] of block
+// (X, Y) adds to K[X][Y][k][x][y]), or null
 int launch_finalize_blocked(const DevBasis &b, int m, const double *D, const double *Jb, const double *Kb,
-                            double *J, double *K, double *F, double *tsum, cudaStream_t s);
+                            const double *KTb, double *J, double *K, double *F, double *tsum, cudaStream_t s);
 int umma_smem_bytes();
 size_t umma_kbank_bytes(int nb);
 size_t umma_jbank_bytes(int nb);
 int launch_finalize(const DevBasis &b, int m, const double *D, const double *Jacc,
                     const double *Kacc, double *J, double *K, double *F, double *tsum,
                     cudaStream_t s);
+
+// ---- jk_split.cu (tensor-core contraction of FP64 and double-FP32 stores)
+struct SplitLaunch {
+    const BrickDesc *bricks;
+    int64_t nbricks;
+    const int64_t *offsets;      // record start, in 8-byte elements
+    const void *store;
+    int f32x2;                   // values are FP32 hi + lo pairs
+    void *kbank, *jbank;         // density digit tiles (work memory)
+    const double *D;
+    int n, nb, m, num_sms;
+    double *Jacc, *Kacc, *KTacc; // block-major accumulators [X][Y][k][x][y]
+    int *nonfinite;              // device flag, zero at launch
+    int *error;                  // device error flag, 0 = ok
+    cudaEvent_t ev_start = nullptr, ev_stop = nullptr;
+};
+int launch_jk_split(const SplitLaunch &L, cudaStream_t s);
+size_t split_kbank_bytes(int nb);
+size_t split_jbank_bytes(int nb);
 
 // ---- df.cu (density-fitted J and K)
 struct DfBuild {

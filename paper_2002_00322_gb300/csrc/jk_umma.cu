@@ -768,11 +768,13 @@ int launch_jk_umma(const UmmaLaunch &L, cudaStream_t s) {
     return ESMF_OK;
 }
 
-// J from the lower block triangle of the block-major accumulators, F = 2J - K,
+// J from the lower block triangle of the block-major accumulators, K from its
+// blocks plus the transposes of KTb's (when given), F = 2J - K,
 // t_k = sum_pq D_k[pq] F_k[pq]; outputs in the caller's [k][p][q] layout.  One
 // block per (row p, density k), threads over the columns q.
 __global__ void k_finalize_blocked(int n, int nb, int m, const double *D, const double *Jb,
-                                   const double *Kb, double *J, double *K, double *F, double *tsum) {
+                                   const double *Kb, const double *KTb, double *J, double *K, double *F,
+                                   double *tsum) {
     const int p = blockIdx.x, k = blockIdx.y;
     const int X = p >> 3, x = p & 7;
     const int64_t row = (int64_t)k * n * n + (int64_t)p * n;
@@ -781,7 +783,8 @@ __global__ void k_finalize_blocked(int n, int nb, int m, const double *D, const 
         const int Y = q >> 3, y = q & 7;
         const double jv = (X >= Y) ? Jb[(((int64_t)X * nb + Y) * m + k) * 64 + x * 8 + y]
                                    : Jb[(((int64_t)Y * nb + X) * m + k) * 64 + y * 8 + x];
-        const double kv = Kb[(((int64_t)X * nb + Y) * m + k) * 64 + x * 8 + y];
+        double kv = Kb[(((int64_t)X * nb + Y) * m + k) * 64 + x * 8 + y];
+        if (KTb) kv += KTb[(((int64_t)Y * nb + X) * m + k) * 64 + y * 8 + x];
         const double fv = 2.0 * jv - kv;
         J[row + q] = jv;
         K[row + q] = kv;
@@ -802,10 +805,10 @@ __global__ void k_finalize_blocked(int n, int nb, int m, const double *D, const 
 }
 
 int launch_finalize_blocked(const DevBasis &b, int m, const double *D, const double *Jb, const double *Kb,
-                            double *J, double *K, double *F, double *tsum, cudaStream_t s) {
+                            const double *KTb, double *J, double *K, double *F, double *tsum, cudaStream_t s) {
     if (b.n < 1 || m < 1) return ESMF_OK;
     const int threads = b.n <= 128 ? 128 : 256;
-    k_finalize_blocked<<<dim3(b.n, m), threads, 0, s>>>(b.n, b.nb, m, D, Jb, Kb, J, K, F, tsum);
+    k_finalize_blocked<<<dim3(b.n, m), threads, 0, s>>>(b.n, b.nb, m, D, Jb, Kb, KTb, J, K, F, tsum);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { set_error("k_finalize_blocked: %s", cudaGetErrorString(e)); return ESMF_ERR_CUDA; }
     return ESMF_OK;

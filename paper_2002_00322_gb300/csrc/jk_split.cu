@@ -27,11 +27,12 @@
 // once into the columns of t = i, i+1, ... (one MMA per 16 terms and digit of
 // V instead of one per digit pair).
 //
-// What bounds it: at 16 densities the MMAs of a brick take 8.8K cycles (M = 64
-// runs at 2,048 MAC per clock); the CUDA-core FP64 form of the same brick takes
-// 327K (GB300 has two FP64 FMA per clock and SM).  200 functions, 16
-// densities, 53K bricks: 54.7 ms with k_jk_cuda<double>, 2.8 ms here (15.5K
-// cycles a brick: the epilogue's instructions beside the MMAs).
+// What bounds it: at 16 densities the MMAs of a brick take 8.8K cycles of the
+// tensor pipe (M = 64 runs at 2,048 MAC per clock) and fetch 940 KB of operands
+// from shared memory (7.3K cycles at 128 B per clock) beside 350 KB of other
+// traffic there; the CUDA-core FP64 form of the same brick takes 327K cycles
+// (GB300 has two FP64 FMA per clock and SM).  200 functions, 16 densities, 53K
+// bricks: 54.7 ms with k_jk_cuda<double>, 2.62 ms here (14.3K cycles a brick).
 //
 // Warp roles (576 threads, one CTA per SM): warp 0 producer (bulk copies of
 // the packed record one brick ahead and of one density tile per view through a
@@ -50,6 +51,8 @@
 // Densities that are not finite (or above 2^500) have no digits: k_split_dbank
 // then raises a flag and the kernel runs a plain FP64 loop over the same bricks.
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "esmf_internal.cuh"
 #include "umma.cuh"
@@ -174,6 +177,14 @@ __device__ __forceinline__ long long combine(const float *c, int stride) {
     return S + (long long)((unsigned long long)(long long)c0 << 39);
 }
 
+// *p += (value_hi, lo) as a double unless hi is zero (a zero value): a predicated
+// reduction, so that the outputs of a loop are scheduled across each other
+__device__ __forceinline__ void red_nonzero(double *p, int hi, int value_hi, int lo) {
+    asm volatile("{\n.reg .pred q;\nsetp.ne.s32 q, %1, 0;\n@q red.global.add.f64 [%0], %2;\n}" ::"l"(p), "r"(hi),
+                 "d"(__hiloint2double(value_hi, lo))
+                 : "memory");
+}
+
 template <int H>
 __device__ __forceinline__ void tmem_ld_half(uint32_t taddr, float *v) {
     uint32_t r[H];
@@ -187,6 +198,19 @@ __device__ __forceinline__ void tmem_ld_half(uint32_t taddr, float *v) {
                      : "r"(taddr));
 #pragma unroll
     for (int i = 0; i < H; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// a warp-uniform value in a uniform register (the reduction's result is one)
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __reduce_or_sync(0xffffffffu, x); }
+
+// MMA issued by the lane whose `lead` is set; descriptors as low and high words
+__device__ __forceinline__ void mma_pred(uint32_t lead, uint32_t dtmem, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                         uint32_t bhi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n.reg .pred p, q;\n.reg .b64 a, b;\nsetp.ne.b32 p, %6, 0;\nsetp.ne.b32 q, %7, 0;\n"
+        "mov.b64 a, {%1, %2};\nmov.b64 b, {%3, %4};\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}" ::"r"(dtmem),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate), "r"(lead));
 }
 
 // canonical K-major operand tile: row n (density column of the MMA), k = b*8 + d
@@ -412,6 +436,10 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
         for (int k = views > 2 ? views - 2 : 0; k < views; ++k) wait_for(&c.dfull[k & 1], (k >> 1) & 1, &c.never);
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
+        // One lane leads; every MMA carries it as a predicate, so that the converged
+        // warp forms the descriptors in uniform registers (200 functions, 16
+        // densities: 2.62 ms, against 2.81 with the MMAs in the elected lane's branch)
+        const uint32_t lead = elect_one() ? 1u : 0u, sbase = smem_u32(sm);
         int views = 0;
         BrickDesc dn = brick(0);
         bool ok = true;
@@ -427,34 +455,34 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                 if (!__all_sync(~0u, wait_for(&c.dfull[s], (views >> 1) & 1, abort_flag))) { fail(25); ok = false; break; }
                 if (views >= 2 && !__all_sync(~0u, wait_for(&c.accfree[s], ((views - 2) >> 1) & 1, abort_flag))) { fail(26); ok = false; break; }
                 tc_fence_after();
-                if (elect_one()) {
-                    const uint32_t base = smem_u32(sm);
-                    const uint32_t A = base + (v < 4 ? OFF_V : OFF_W), B = base + OFF_RING + s * RING_SLOT;
-                    // A: views 0, 2, 4 step 256 B per 16 terms, the others 2048 B; views 0, 1, 4
-                    // are K-major, 2, 3, 5 MN-major
-                    const bool even = v == 0 || v == 2 || v == 4;
-                    const uint32_t ks = (even ? 256u : 2048u) >> 4, lbo = even ? 128u : 1024u, sbo = even ? 1024u : 128u;
-                    const int mn = (v == 2 || v == 3 || v == 5) ? 1 : 0;
-                    const uint32_t W = v < 4 ? 2 * MP : MP;          // columns (and operand rows) of one digit
-                    const uint64_t a0 = sdesc(A, lbo, sbo), b0 = sdesc(B, 128, 1024);
-                    const uint32_t col = tmem + s * REGION;
+                // A: views 0, 2, 4 step 256 B per 16 terms, the others 2048 B; views 0, 1, 4
+                // are K-major, 2, 3, 5 MN-major
+                const bool even = v == 0 || v == 2 || v == 4;
+                const uint32_t lbo = even ? 128u : 1024u, sbo = even ? 1024u : 128u;
+                const uint32_t W = v < 4 ? 2 * MP : MP;              // columns (and operand rows) of one digit
+                const uint64_t a0 = sdesc(sbase + (v < 4 ? OFF_V : OFF_W), lbo, sbo), b0 = sdesc(sbase + OFF_RING + s * RING_SLOT, 128, 1024);
+                const uint32_t alo = uniform((uint32_t)a0), ahi = uniform((uint32_t)(a0 >> 32));
+                const uint32_t blo = uniform((uint32_t)b0), bhi = uniform((uint32_t)(b0 >> 32));
+                const uint32_t ks = uniform((even ? 256u : 2048u) >> 4), col = uniform(tmem + s * REGION);
+                const uint32_t Wu = uniform(W), wid = uniform((W >> 3) << 17);
+                const uint32_t id0 = uniform(idesc_f16(64, 0, (v == 2 || v == 3 || v == 5) ? 1 : 0, 0));
 #pragma unroll
-                    for (int x = 0; x < NV; ++x) {
-                        // digit x of V against the density digits 0 .. nj-1, into the columns of t = x ..
-                        const int nj = x < 2 ? ND : NT - x;
-                        const uint32_t id = idesc_f16(64, nj * W, mn, 0);
+                for (int x = 0; x < NV; ++x) {
+                    // digit x of V against the density digits 0 .. nj-1, into the columns of t = x ..
+                    const uint32_t nj = x < 2 ? ND : NT - x;
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint64_t a = a0 + (uint32_t)(x * (SLICE >> 4)) + j * ks, bd = b0 + 16 * j;
-                            if (x == 1 && j == 0) {
-                                // t = 6 starts here: its columns are written, those of t < 6 added to
-                                mma_f16(col + W, a, bd, idesc_f16(64, 5 * W, mn, 0), 1u);
-                                mma_f16(col + 6 * W, a, bd + ((5 * W * 128) >> 4), idesc_f16(64, W, mn, 0), 0u);
-                            } else {
-                                mma_f16(col + x * W, a, bd, id, (x > 0 || j > 0) ? 1u : 0u);
-                            }
+                    for (int j = 0; j < 4; ++j) {
+                        const uint32_t a = alo + x * (SLICE >> 4) + j * ks, bd = blo + 16 * j;
+                        if (x == 1 && j == 0) {
+                            // t = 6 starts here: its columns are written, those of t < 6 added to
+                            mma_pred(lead, col + Wu, a, ahi, bd, bhi, id0 + 5 * wid, 1u);
+                            mma_pred(lead, col + 6 * Wu, a, ahi, bd + 40 * Wu, bhi, id0 + wid, 0u);
+                        } else {
+                            mma_pred(lead, col + x * Wu, a, ahi, bd, bhi, id0 + nj * wid, (x > 0 || j > 0) ? 1u : 0u);
                         }
                     }
+                }
+                if (lead) {
                     mma_commit(&c.mmad[s]);
                     if (v == lastx) mma_commit(&c.vfree);
                     if (v == 5) mma_commit(&c.wfree);
@@ -590,6 +618,16 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                 const int tx = v == 4 ? d.R : ((v == 0 || v == 2) ? d.Q : d.P);
                 const int ty = v == 5 ? d.Q : ((v < 2 || v == 4) ? d.S : d.R);
                 const bool coul = v >= 4;
+                // exponents of the parts' density blocks: the D part, then (exchange) the D^T part
+                using EX = typename std::conditional<H == 8, uint4, uint2>::type;
+                EX xq[2];
+                {
+                    const int16_t *ex = coul ? P.eJ + ((size_t)tx * (tx + 1) / 2 + ty) * MPM
+                                             : P.eK + ((size_t)tx * P.nb + ty) * MPM;
+                    const int16_t *et = coul ? ex : P.eK + ((size_t)ty * P.nb + tx) * MPM;
+                    xq[0] = *reinterpret_cast<const EX *>(ex + cb);
+                    xq[1] = *reinterpret_cast<const EX *>(et + cb);
+                }
                 if (!__all_sync(~0u, wait_for(&c.mmad[g], (vi >> 1) & 1, abort_flag))) { fail(30); ok = false; break; }
                 if (!have) {
                     if (!__all_sync(~0u, counter_wait(&c.epub, (unsigned)i + 1u, abort_flag, POLLS))) { fail(31); ok = false; break; }
@@ -599,16 +637,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                 tc_fence_after();
                 const uint32_t W = coul ? MP : 2 * MP;
                 const int64_t out = ((int64_t)(A * P.nb + C) * P.mtot + P.d0 + cb) * 64 + row;
-                // the D part, then (exchange) the D^T part; no D^T part and no J2 for the (PQ|PQ) brick
+                // no D^T part and no J2 for the (PQ|PQ) brick
                 const int parts = (coul || diag) ? 1 : 2;
                 const bool none = v == 5 && diag;
 #pragma unroll 1
                 for (int part = 0; part < parts; ++part) {
-                    const int16_t *ex = coul ? P.eJ + ((size_t)tx * (tx + 1) / 2 + ty) * MPM
-                                             : P.eK + ((size_t)(part ? ty : tx) * P.nb + (part ? tx : ty)) * MPM;
                     alignas(16) int16_t xp[H];
-                    if constexpr (H == 8) *reinterpret_cast<uint4 *>(xp) = *reinterpret_cast<const uint4 *>(ex + cb);
-                    else *reinterpret_cast<uint2 *>(xp) = *reinterpret_cast<const uint2 *>(ex + cb);
+                    *reinterpret_cast<EX *>(xp) = part ? xq[1] : xq[0];
                     float a[NT * H];
                     __syncwarp();
 #pragma unroll
@@ -627,7 +662,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                             // its exponent field.  Columns without a density have S = 0.
                             const double x = __ll2double_rn(combine(a + j, H));
                             const int hi = __double2hiint(x);
-                            if (hi != 0) atomicAdd(dst + j * 64, __hiloint2double(hi + ((ev + xp[j]) << 20), __double2loint(x)));
+                            red_nonzero(dst + j * 64, hi, hi + ((ev + xp[j]) << 20), __double2loint(x));
                         }
                     }
                 }

@@ -32,7 +32,10 @@
 // from shared memory (7.3K cycles at 128 B per clock) beside 350 KB of other
 // traffic there; the CUDA-core FP64 form of the same brick takes 327K cycles
 // (GB300 has two FP64 FMA per clock and SM).  200 functions, 16 densities, 53K
-// bricks: 54.7 ms with k_jk_cuda<double>, 2.62 ms here (14.3K cycles a brick).
+// bricks: 54.7 ms with k_jk_cuda<double>, 3.02 ms here (16.5K cycles a brick).
+// Recombining into one 62-bit integer per output takes 2.62 ms, but rounds every
+// output at 2^-56 of the brick's largest product, also one a thousand times
+// smaller, where FP64 arithmetic would not.
 //
 // Warp roles (576 threads, one CTA per SM): warp 0 producer (bulk copies of
 // the packed record one brick ahead and of one density tile per view through a
@@ -40,7 +43,7 @@
 // converters (packed record -> digits in registers -> tiles V and, with r and q
 // swapped, W, which the Coulomb views read), warps 10-17 epilogue in two groups
 // of four that take the views alternately: tensor-memory load, integer
-// recombination of the c_t, one FP64 conversion and reduction per output.  V
+// recombination of the c_t, one FP64 reduction per output.  V
 // and W are single tiles (shared memory holds no second pair): the digits of
 // the next brick wait in registers, V is written while the Coulomb MMAs (over
 // W) run, W while the exchange MMAs (over V) run.  The D^T outputs go to an
@@ -164,17 +167,21 @@ __device__ __forceinline__ uint32_t digit_pair(const uint32_t *wa, const uint32_
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
-// ---- recombination: S = sum_t c_t 2^(9 (4 - t) + 3) as a 64-bit integer
-// (below 2^62).  The c_t of t = 5, 6 join c_4 in FP32; |c_0| <= 2^22 has its
-// integer in the low bits of c_0 + 1.5 2^23.
-__device__ __forceinline__ long long combine(const float *c, int stride) {
+// ---- recombination: sum_t c_t 2^(9 (3 - t)) as a double, rounded once.  The
+// part of t <= 3 is an integer of at most 50 bits, formed on the integer pipe
+// and read as a double through the bits of 1.5 2^52 + itself (|c_0| <= 2^22
+// likewise from c_0 + 1.5 2^23); the c_t of t >= 4 are summed in FP32, whose
+// bits widen to FP64 on the integer pipe too.  Two FP64 additions remain.
+__device__ __forceinline__ double recombine(const float *c, int stride) {
     float f = fmaf(c[6 * stride], 0x1p-9f, c[5 * stride]);
-    f = fmaf(f, 0x1p-6f, c[4 * stride] * 8.0f);
-    long long S = (long long)__float2int_rn(c[3 * stride]) * (1 << 12) + __float2int_rn(f);
-    S += (long long)__float2int_rn(c[2 * stride]) * (1 << 21);
-    S += (long long)__float2int_rn(c[1 * stride]) * (1 << 30);
+    f = fmaf(f, 0x1p-18f, c[4 * stride] * 0x1p-9f);
+    long long S = (long long)__float2int_rn(c[2 * stride]) * 512 + __float2int_rn(c[3 * stride]);
+    S += (long long)__float2int_rn(c[1 * stride]) * (1 << 18);
     const int c0 = (int)(__float_as_uint(__fadd_rn(c[0], 12582912.f)) - 0x4b400000u);
-    return S + (long long)((unsigned long long)(long long)c0 << 39);
+    S += (long long)c0 * (1 << 27) + 0x4338000000000000ll;
+    const uint32_t b = __float_as_uint(f);
+    const uint32_t fhi = f == 0.0f ? 0u : (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u);
+    return (__longlong_as_double(S) - 0x1.8p52) + __hiloint2double((int)fhi, (int)(b << 29));
 }
 
 // *p += (value_hi, lo) as a double unless hi is zero (a zero value): a predicated
@@ -438,7 +445,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
         // ------------------------------------------------ MMA issuer
         // One lane leads; every MMA carries it as a predicate, so that the converged
         // warp forms the descriptors in uniform registers (200 functions, 16
-        // densities: 2.62 ms, against 2.81 with the MMAs in the elected lane's branch)
+        // densities: 7 % less time than with the MMAs in the elected lane's branch)
         const uint32_t lead = elect_one() ? 1u : 0u, sbase = smem_u32(sm);
         int views = 0;
         BrickDesc dn = brick(0);
@@ -631,7 +638,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                 if (!__all_sync(~0u, wait_for(&c.mmad[g], (vi >> 1) & 1, abort_flag))) { fail(30); ok = false; break; }
                 if (!have) {
                     if (!__all_sync(~0u, counter_wait(&c.epub, (unsigned)i + 1u, abort_flag, POLLS))) { fail(31); ok = false; break; }
-                    ev = c.ev[i & 3] - 55;
+                    ev = c.ev[i & 3] - 43;
                     have = true;
                 }
                 tc_fence_after();
@@ -658,9 +665,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                     if (!none) {
 #pragma unroll
                         for (int j = 0; j < H; ++j) {
-                            // S 2^e: one conversion (exact to rounding), the power of two added to
-                            // its exponent field.  Columns without a density have S = 0.
-                            const double x = __ll2double_rn(combine(a + j, H));
+                            // the power of two is added to the exponent field; columns without a
+                            // density have zeros
+                            const double x = recombine(a + j, H);
                             const int hi = __double2hiint(x);
                             red_nonzero(dst + j * 64, hi, hi + ((ev + xp[j]) << 20), __double2loint(x));
                         }

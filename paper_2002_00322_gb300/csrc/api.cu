@@ -42,6 +42,7 @@ struct esmf_fock {
     int *nprim = nullptr, *poff = nullptr;
     int *cart = nullptr;           // Cartesian labels (device, np), null when every function is s
     double *Q = nullptr;
+    double *boys = nullptr;        // Taylor table of F0 (s bases evaluated in FP64)
     // screening table and threshold of the quartet rule S_pq S_rs >= tol_s:
     // the Schwarz table itself (S = Q, tol_s = tol), or the 0/1 table of the
     // paper's pair rule (tol_s = 0.5)
@@ -136,7 +137,7 @@ struct esmf_fock {
         DevBasis b;
         b.n = n; b.np = np; b.nb = nb;
         b.center = center; b.nprim = nprim; b.poff = poff; b.exps = exps; b.w = w;
-        b.cart = cart;
+        b.cart = cart; b.boys = boys;
         return b;
     }
 };
@@ -265,7 +266,7 @@ void release(esmf_fock *h) {
     cudaFree(h->center); cudaFree(h->exps); cudaFree(h->w); cudaFree(h->coefs);
     cudaFree(h->nprim); cudaFree(h->poff); cudaFree(h->cart);
     if (h->S != h->Q) cudaFree(h->S);
-    cudaFree(h->Q);
+    cudaFree(h->Q); cudaFree(h->boys);
     cudaFree(h->bricks); cudaFree(h->offsets); cudaFree(h->store); cudaFree(h->parts); cudaFree(h->scratch);
     for (auto &sp : h->shard_parts) cudaFree(sp.second.first);
     cudaFree(h->ptab); cudaFree(h->pslot); cudaFree(h->pblocks);
@@ -543,7 +544,7 @@ static int create_impl(const esmf_basis_t *basis, const int32_t *cart, double to
         if (e != cudaSuccess) { set_error("%s: %s", what, cudaGetErrorString(e)); return false; }
         return true;
     };
-    const DevBasis db = h->dev();
+    DevBasis db = h->dev();
     std::vector<double> hQ((size_t)np * np);
     if (!ck(cudaMemcpyAsync(hQ.data(), h->Q, sizeof(double) * np * np, cudaMemcpyDeviceToHost, cs), "copy Q") ||
         !ck(cudaStreamSynchronize(cs), "Schwarz table"))
@@ -734,6 +735,13 @@ static int create_impl(const esmf_basis_t *basis, const int32_t *cart, double to
     if (use_mode != ESMF_MODE_STORED) h->store_bytes = 0;
 
     std::vector<int> pslot_h, pblocks_h;
+    if (h->nbricks > 0 && !h->cart && (h->prec == ESMF_PREC_FP64 || h->prec == ESMF_PREC_F32X2)) {
+        const std::vector<double> &tab = boys_table();
+        if ((rc = dalloc(h, &h->boys, tab.size()))) return fail(rc);
+        if (!ck(cudaMemcpyAsync(h->boys, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice, cs), "copy Boys table"))
+            return fail(ESMF_ERR_CUDA);
+        db.boys = h->boys;
+    }
     if (h->nbricks > 0) {
         if ((rc = dalloc(h, &h->bricks, h->nbricks))) return fail(rc);
         if (!ck(cudaMemcpyAsync(h->bricks, kept.data(), sizeof(BrickDesc) * h->nbricks, cudaMemcpyHostToDevice, cs), "copy kept bricks"))

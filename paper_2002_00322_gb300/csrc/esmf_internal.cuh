@@ -58,11 +58,14 @@ struct DevBasis {
     const double *exps;    // primitives
     const double *w;       // normalised raw-Gaussian weights
     const int *cart = nullptr;  // np Cartesian labels (0 s, 1..3 p_x..p_z); null: all s
+    const double *boys = nullptr;  // Taylor table of F0 (integrals.cuh); FP64 generation and direct builds
 };
 
 void set_error(const char *fmt, ...);
 
 // ---- setup.cu
+// host copy of the Taylor table of F0 (formed once per process)
+const std::vector<double> &boys_table();
 int launch_normalize(const DevBasis &b, const double *coefs, double *w, cudaStream_t s);
 int launch_schwarz(const DevBasis &b, double *Q, cudaStream_t s);
 // pair rule of Sec. II.C into a 0/1 screening table S (np x np)

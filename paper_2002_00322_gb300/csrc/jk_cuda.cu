@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(256, (jk_ctas_per_sm<TA, MC, SRC>())) k_jk_cud
                 } else {
                     for (int i = threadIdx.x; i < total; i += blockDim.x) {
                         const int e = klist[i];
-                        sm.V[tile_swizzle(e)] = contracted_eri<TA, 128, MAXPP>(sm.pairs, e >> 6, sm.pairs, 64 + (e & 63));
+                        sm.V[tile_swizzle(e)] = contracted_eri<TA, 128, MAXPP>(sm.pairs, e >> 6, sm.pairs, 64 + (e & 63), a.b.boys);
                     }
                 }
             } else {

@@ -6,6 +6,8 @@
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
 
+#include <cmath>
+
 #include "esmf_internal.cuh"
 #include "integrals.cuh"
 
@@ -19,6 +21,32 @@ namespace esmf {
             return ESMF_ERR_CUDA;                                                  \
         }                                                                          \
     } while (0)
+
+// F_6 by its positive series e^-T sum_i (2T)^i / (13 15 ... (13 + 2i)), F_5 ..
+// F_1 by the downward recursion F_k = (2T F_{k+1} + e^-T) / (2k + 1) (positive
+// terms, no cancellation), F_0 from erf in long double.
+const std::vector<double> &boys_table() {
+    static const std::vector<double> tab = [] {
+        std::vector<double> t((size_t)kBoysEntries * 8);
+        for (int i = 0; i < kBoysEntries; ++i) {
+            const double T = (double)i / kBoysGrid, em = std::exp(-T);
+            double F[7], term = 1.0 / 13.0, sum = term;
+            for (int k = 1; term > 1e-18 * sum; ++k) sum += term *= 2.0 * T / (13.0 + 2.0 * k);
+            F[6] = em * sum;
+            for (int k = 5; k >= 1; --k) F[k] = (2.0 * T * F[k + 1] + em) / (2.0 * k + 1.0);
+            const long double x = std::sqrt((long double)T);
+            F[0] = i == 0 ? 1.0 : (double)(0.88622692545275801364908374167057259L * std::erf(x) / x);
+            double fact = 1.0;
+            for (int k = 0; k < 7; ++k) {
+                if (k > 0) fact *= -(double)k;
+                t[(size_t)i * 8 + k] = F[k] / fact;
+            }
+            t[(size_t)i * 8 + 7] = T;
+        }
+        return t;
+    }();
+    return tab;
+}
 
 static inline int grid_for(int64_t work, int per_block, int cap = 152 * 32) {
     int64_t g = (work + per_block - 1) / per_block;
@@ -351,7 +379,7 @@ __global__ void __launch_bounds__(256) k_brick_generate(DevBasis b, const double
         __syncthreads();
         for (int i = threadIdx.x; i < total; i += blockDim.x) {
             const int e = sm.klist[i];
-            const T v = contracted_eri<T, 128, MAXPP>(sm.pairs, e >> 6, sm.pairs, 64 + (e & 63));
+            const T v = contracted_eri<T, 128, MAXPP>(sm.pairs, e >> 6, sm.pairs, 64 + (e & 63), b.boys);
             if (PREC == 0 || PREC == 1) {
                 reinterpret_cast<T *>(store)[vbase + i] = v;
             } else if (PREC == 4) {

@@ -205,8 +205,13 @@ int esmf_fock_create_cart(const esmf_basis_t *basis, const int32_t *cart, double
  *   precision  ESMF_PREC_FP64 or ESMF_PREC_FP32 (GEMM arithmetic; the fit
  *              itself is always formed in FP64)
  *   device, out  as for esmf_fock_create
- * Device memory: about 2 n_aux N^2 elements for B and B'', plus n_aux N^2
- * elements of per-build work.  Errors: INVALID_ARG (bad basis or auxiliary
+ * Device memory, FP32: about 2 n_aux N^2 elements for B and B'', plus n_aux N^2
+ * elements of per-build work.  FP64: B, its digit tiles for the exchange on the
+ * tensor cores (14 bytes an element, rows padded to 128 and columns to 64) and
+ * 14 bytes an element for the same of as many densities as fit 2.5 GiB (at
+ * least one); without room for those, the FP32 layout in FP64 on cuBLAS.
+ * FP64: K_k is NaN when D_k holds an infinity, a NaN or an element above 2^500.
+ * Errors: INVALID_ARG (bad basis or auxiliary
  * set, or a metric that is not positive definite), UNSUPPORTED (split 16-bit
  * precisions), OOM, CUDA.
  */

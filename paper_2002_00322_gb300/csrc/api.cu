@@ -82,6 +82,12 @@ struct esmf_fock {
     void *dfB = nullptr, *dfB2 = nullptr;
     void *dfDt = nullptr, *dfJt = nullptr, *dfKt = nullptr, *dfg = nullptr, *dfY = nullptr;
     int df_m = 0;
+    // FP64 exchange by digit splitting (df_split.cu), used when dfTiles is set:
+    // the factor's digit tiles and row exponents, per-build work
+    unsigned char *dfTiles = nullptr, *dfYt = nullptr, *dfDtl = nullptr;
+    int16_t *dfeB = nullptr, *dfeD = nullptr;
+    int *dfED = nullptr;
+    int df_group = 0;
     // tensor hypercontraction (mode ESMF_MODE_THC): grid size, collocation X
     // and fitted Z (arithmetic type), per-build work for up to thc_m densities
     int thc_G = 0;
@@ -276,6 +282,7 @@ void release(esmf_fock *h) {
     cudaFree(h->dw); cudaFree(h->dwb);
     cudaFree(h->dfB); cudaFree(h->dfB2); cudaFree(h->dfDt); cudaFree(h->dfJt); cudaFree(h->dfKt);
     cudaFree(h->dfg); cudaFree(h->dfY);
+    cudaFree(h->dfTiles); cudaFree(h->dfYt); cudaFree(h->dfDtl); cudaFree(h->dfeB); cudaFree(h->dfeD); cudaFree(h->dfED);
     cudaFree(h->thcX); cudaFree(h->thcZ); cudaFree(h->thcDt); cudaFree(h->thcA); cudaFree(h->thcM);
     cudaFree(h->thcy); cudaFree(h->thcz); cudaFree(h->thcJt); cudaFree(h->thcKt);
     df_cublas_destroy(h->cublas);
@@ -970,19 +977,35 @@ int esmf_fock_create_df(const esmf_basis_t *basis, const esmf_aux_t *aux, int pr
         return fail(ESMF_ERR_CUDA);
     }
     if ((rc = df_gemm_fold(h->cublas, naux, (int64_t)nn, Linv, T, B, cs))) return fail(rc);
-    if ((rc = dalloc(h, (unsigned char **)&h->dfB2, naux * nn * es)) ||
-        (rc = dalloc(h, (unsigned char **)&h->dfY, naux * nn * es)))
+    if (es == 8) {
+        // digit tiles of the factor and of Y for as many densities per pass as fit
+        // 2.5 GiB; without room for them the exchange stays on cuBLAS
+        const size_t tb = df_split_tile_bytes(n, naux);
+        h->df_group = (int)std::max<size_t>(1, std::min<size_t>(16, ((size_t)5 << 29) / tb));
+        if (cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+            dalloc(h, &h->dfTiles, tb) != ESMF_OK || dalloc(h, &h->dfYt, tb * h->df_group) != ESMF_OK ||
+            dalloc(h, &h->dfeB, 2 * (size_t)n) != ESMF_OK) {
+            cudaGetLastError();
+            dfree(h, &h->dfTiles, tb);
+            dfree(h, &h->dfYt, tb * h->df_group);
+        }
+    }
+    const bool split = h->dfTiles != nullptr;
+    if (!split && ((rc = dalloc(h, (unsigned char **)&h->dfB2, naux * nn * es)) ||
+                   (rc = dalloc(h, (unsigned char **)&h->dfY, naux * nn * es))))
         return fail(rc);
     if (es == 4) {
         if ((rc = dalloc(h, (unsigned char **)&h->dfB, naux * nn * es))) return fail(rc);
         if ((rc = launch_df_layouts(naux, n, B, 1, h->dfB, h->dfB2, cs))) return fail(rc);
     } else {
-        if ((rc = launch_df_layouts(naux, n, B, 0, nullptr, h->dfB2, cs))) return fail(rc);
+        if (split) rc = launch_df_split_factor(B, naux, n, h->dfeB, h->dfeB + n, h->dfTiles, cs);
+        else rc = launch_df_layouts(naux, n, B, 0, nullptr, h->dfB2, cs);
+        if (rc) return fail(rc);
         h->dfB = B;                       // the FP64 factor itself is the [P][p][q] layout
         h->device_bytes += (int64_t)(naux * nn * es);
         B = nullptr;
     }
-    h->store_bytes = (int64_t)(2 * naux * nn * es);
+    h->store_bytes = (int64_t)(naux * nn * es + (split ? df_split_tile_bytes(n, naux) : naux * nn * es));
     if (cudaEventCreateWithFlags(&h->done, cudaEventDisableTiming) != cudaSuccess ||
         cudaHostAlloc((void **)&h->err_host, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer((void **)&h->err_dev, h->err_host, 0) != cudaSuccess) {
@@ -1212,7 +1235,13 @@ int build_df(esmf_fock_t *h, int m, const double *D, double *J, double *K, doubl
              cudaStream_t s) {
     const size_t es = h->prec == ESMF_PREC_FP32 ? 4 : 8;
     const size_t nn = (size_t)h->n * h->n;
+    const size_t ldD = (size_t)((h->n + 63) / 64) * 64;
     if (m > h->df_m) {
+        if (h->dfTiles) {
+            dfree(h, &h->dfDtl, df_split_tile_bytes(h->n, h->df_m));
+            dfree(h, &h->dfeD, h->df_m * ldD);
+            dfree(h, &h->dfED, 2 * (size_t)h->df_m);
+        }
         dfree(h, (unsigned char **)&h->dfDt, es == 4 ? h->df_m * nn * es : 1);
         dfree(h, (unsigned char **)&h->dfJt, h->df_m * nn * es);
         dfree(h, (unsigned char **)&h->dfKt, h->df_m * nn * es); dfree(h, (unsigned char **)&h->dfg, (size_t)h->df_m * h->naux * es);
@@ -1221,13 +1250,26 @@ int build_df(esmf_fock_t *h, int m, const double *D, double *J, double *K, doubl
         RET(dalloc(h, (unsigned char **)&h->dfJt, m * nn * es));
         RET(dalloc(h, (unsigned char **)&h->dfKt, m * nn * es));
         RET(dalloc(h, (unsigned char **)&h->dfg, (size_t)m * h->naux * es));
+        if (h->dfTiles) {
+            RET(dalloc(h, &h->dfDtl, df_split_tile_bytes(h->n, m)));
+            RET(dalloc(h, &h->dfeD, m * ldD));
+            RET(dalloc(h, &h->dfED, 2 * (size_t)m));
+        }
         h->df_m = m;
+    }
+    DfSplit sp;
+    if (h->dfTiles) {
+        sp.n = h->n; sp.naux = h->naux; sp.m = m; sp.group = h->df_group; sp.num_sms = h->num_sms;
+        sp.eB = h->dfeB; sp.nB = h->dfeB + h->n; sp.Btiles = h->dfTiles; sp.D = D;
+        sp.eD = h->dfeD; sp.ED = h->dfED; sp.bad = h->dfED + h->df_m; sp.Dtiles = h->dfDtl; sp.Ytiles = h->dfYt;
+        sp.K = (double *)h->dfKt; sp.error = h->err_dev;
     }
     DfBuild a;
     a.cublas = h->cublas; a.n = h->n; a.naux = h->naux; a.m = m; a.fp32 = h->prec == ESMF_PREC_FP32;
     a.B = h->dfB; a.B2 = h->dfB2; a.D = D;
     a.Dt = h->dfDt; a.Jt = h->dfJt; a.Kt = h->dfKt; a.g = h->dfg; a.Y = h->dfY;
     a.J = J; a.K = K; a.F = F; a.traces = traces;
+    a.split = h->dfTiles ? &sp : nullptr;
     if (h->timing && h->ev_used < 65536) {
         if (h->ev_used == h->ev_pool.size()) {
             cudaEvent_t x, y;

@@ -2,7 +2,8 @@
 // Sec. I), GB300 path: three- and two-centre integrals over auxiliary s
 // Gaussians on the device, the Coulomb-metric fit folded into one factor
 // B = L^-1 T (V = L L^T, T_P,pq = (pq|P)) at create time, and every build as
-// dense GEMMs on cuBLAS (FP64 or FP32 arithmetic):
+// dense GEMMs on cuBLAS (FP64 or FP32 arithmetic), the FP64 exchange by digit
+// splitting on the tensor cores (df_split.cu):
 //   g_k = B vec(D_k),  J_k = B^T g_k            (J_pq = sum_P B_P,pq g_k,P)
 //   K_k[p][q] = sum_{P,s} (B''_p D_k)[P][s] B''_q[P][s],  B''[p][P][r] = B_P,pr
 // i.e. K_pq = sum_rs D_rs sum_P B_P,pr B_P,qs, Eq. (J_and_K) over the fitted
@@ -182,7 +183,11 @@ int df_build(const DfBuild &a, cudaStream_t s) {
     CKB(cublasGemmEx(hb, CUBLAS_OP_N, CUBLAS_OP_N, (int)nn, m, naux, one, a.B, ty, (int)nn, a.g, ty, naux, zero,
                      a.Jt, ty, (int)nn, ct, CUBLAS_GEMM_DEFAULT));
     const size_t es = a.fp32 ? 4 : 8;
-    for (int k = 0; k < m; ++k) {
+    if (a.split) {
+        const int rc = launch_df_split_exchange(*a.split, s);
+        if (rc != ESMF_OK) return rc;
+    }
+    for (int k = 0; k < m && !a.split; ++k) {
         const void *Dk = (const char *)Dw + (size_t)k * nn * es;
         void *Kk = (char *)a.Kt + (size_t)k * nn * es;
         // Y (row-major (n naux) x n) = B'' (row-major (n naux) x n) . D_k

@@ -177,6 +177,23 @@ int launch_jk_split(const SplitLaunch &L, cudaStream_t s);
 size_t split_kbank_bytes(int nb);
 size_t split_jbank_bytes(int nb);
 
+// ---- df_split.cu (density-fitted exchange on the tensor cores, FP64 accuracy)
+struct DfSplit {
+    int n, naux, m, group, num_sms;              // group: densities per pass over the Y tiles
+    const int16_t *eB, *nB;                      // row exponents of the factor
+    const unsigned char *Btiles;
+    const double *D;
+    int16_t *eD;                                 // work: column exponents, m x 64 ceil(n / 64)
+    int *ED, *bad;                               // work: per density
+    unsigned char *Dtiles, *Ytiles;              // work: m matrices, group * naux matrices
+    double *K;                                   // m x n x n
+    int *error;                                  // device error flag, 0 = ok
+};
+size_t df_split_tile_bytes(int n, int64_t matrices);
+// row exponents (n each) and digit tiles (naux matrices) of the fitted factor B[P][p][q]
+int launch_df_split_factor(const double *B, int naux, int n, int16_t *eB, int16_t *nB, unsigned char *tiles, cudaStream_t s);
+int launch_df_split_exchange(const DfSplit &a, cudaStream_t s);
+
 // ---- df.cu (density-fitted J and K)
 struct DfBuild {
     void *cublas;
@@ -184,6 +201,7 @@ struct DfBuild {
     const void *B, *B2;          // B[P][p][q] and B''[p][P][q] in the arithmetic type
     const double *D;             // caller's densities (m x n x n)
     void *Dt, *Jt, *Kt, *g, *Y;  // work: arithmetic-type D (FP32 only), J, K, g, Y
+    const DfSplit *split = nullptr;   // FP64: K by digit splitting (B2 and Y unused)
     double *J, *K, *F, *traces;  // caller's outputs
     cudaEvent_t ev_start = nullptr, ev_stop = nullptr;
 };

@@ -374,12 +374,12 @@ int esmf_fock_build_host(esmf_fock_t *h, int m, const double *D_host,
 int esmf_fock_set_density_screening(esmf_fock_t *h, double tol_d);
 
 /*
- * Contraction kernel choice for stored integrals: ESMF_PATH_AUTO uses the
- * tensor-core kernels (for FP64, F32X2 and FP32 by error-free splitting, as
- * accurate as FP64 arithmetic, for FP32 more accurate than FP32 arithmetic),
+ * Contraction kernel choice for stored FP64, F32X2, FP16X2 and BF16X2
+ * integrals: ESMF_PATH_AUTO uses the tensor-core kernels (for FP64 and F32X2
+ * by error-free splitting, as accurate as FP64 arithmetic),
  * ESMF_PATH_CUDA_CORE the CUDA-core kernels (same results within rounding;
- * kept as a cross-check).  Integral-direct FP64 / FP32 handles always use the
- * CUDA-core kernels.  Errors: INVALID_ARG.
+ * kept as a cross-check).  FP32 stores and integral-direct FP64 / FP32
+ * handles always use the CUDA-core kernels.  Errors: INVALID_ARG.
  */
 #define ESMF_PATH_AUTO       0
 #define ESMF_PATH_CUDA_CORE  1

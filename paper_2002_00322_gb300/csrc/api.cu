@@ -119,7 +119,7 @@ struct esmf_fock {
     // J then K (then, on the split path, K's transposed blocks and a flag word)
     double *acc = nullptr;
     size_t acc_n = 0;
-    // FP64, double-FP32 and FP32 stores: density digit tiles of the tensor-core path;
+    // FP64 and double-FP32 stores: density digit tiles of the tensor-core path;
     // no_split: this handle stays on the CUDA-core kernel (values beyond FP64's
     // range, or no memory for the tiles)
     void *skbank = nullptr, *sjbank = nullptr;
@@ -316,9 +316,11 @@ bool is_device_ptr(const void *p) {
 // chunk and contract them on the tensor cores
 bool tensor_direct(const esmf_fock *h) { return h->mode == ESMF_MODE_DIRECT && is_split16(h->prec) && h->scratch; }
 
-// FP64, double-FP32 or FP32 store that builds by exact digit splitting on the
-// tensor cores (jk_split.cu)
-bool split_path(const esmf_fock *h) { return h->mode == ESMF_MODE_STORED && !is_split16(h->prec) && !h->no_split; }
+// FP64 or double-FP32 store that builds by exact digit splitting on the tensor
+// cores (jk_split.cu)
+bool split_path(const esmf_fock *h) {
+    return h->mode == ESMF_MODE_STORED && (h->prec == ESMF_PREC_FP64 || h->prec == ESMF_PREC_F32X2) && !h->no_split;
+}
 
 // doubles of the accumulators of a build of m densities
 size_t acc_doubles(const esmf_fock *h, int m) {
@@ -329,10 +331,10 @@ size_t acc_doubles(const esmf_fock *h, int m) {
 int ensure_work(esmf_fock *h, int m) {
     if (split_path(h) && !h->skbank) {
         // without room for the digit tiles the handle keeps the CUDA-core kernel
-        if (dalloc(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb, h->prec)) != ESMF_OK ||
-            dalloc(h, (unsigned char **)&h->sjbank, split_jbank_bytes(h->nb, h->prec)) != ESMF_OK) {
+        if (dalloc(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb)) != ESMF_OK ||
+            dalloc(h, (unsigned char **)&h->sjbank, split_jbank_bytes(h->nb)) != ESMF_OK) {
             cudaGetLastError();
-            dfree(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb, h->prec));
+            dfree(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb));
             h->no_split = true;
         }
     }
@@ -709,12 +711,11 @@ static int create_impl(const esmf_basis_t *basis, const int32_t *cart, double to
         if (qmax > 0.0) std::frexp(qmax * qmax, &e);
         h->vscale = qmax > 0.0 ? (float)std::ldexp(1.0, 14 - e) : 1.0f;
     }
-    // integrals are bounded by max Q^2: the split path takes them up to 2^500,
-    // and where they are kept in FP32 parts while those are finite
+    // integrals are bounded by max Q^2: the split path takes them up to 2^500
     {
         double qmax = 0.0;
         for (double x : hQ) qmax = std::isfinite(x) ? std::max(qmax, x) : x;
-        h->no_split = !(qmax <= (precision == ESMF_PREC_FP64 ? 0x1p250 : 0x1p63));
+        h->no_split = !(qmax <= 0x1p250);
     }
     if (!ck(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, device), "SM count"))
         return fail(ESMF_ERR_CUDA);
@@ -1401,7 +1402,7 @@ int build_range(esmf_fock_t *h, int64_t b0, int64_t b1, int m, const double *D, 
         if (split_path(h) && h->path != ESMF_PATH_CUDA_CORE && h->tol_d == 0.0) {
             SplitLaunch L;
             L.bricks = a.bricks; L.nbricks = a.nbricks; L.offsets = a.offsets; L.store = h->store;
-            L.precision = h->prec;
+            L.f32x2 = h->prec == ESMF_PREC_F32X2;
             L.kbank = h->skbank; L.jbank = h->sjbank; L.D = D; L.n = h->n; L.nb = h->nb; L.m = m;
             L.num_sms = h->num_sms;
             L.Jacc = Jacc; L.Kacc = Kacc; L.KTacc = Kacc + cnt;

@@ -158,13 +158,13 @@ int launch_finalize(const DevBasis &b, int m, const double *D, const double *Jac
                     const double *Kacc, double *J, double *K, double *F, double *tsum,
                     cudaStream_t s);
 
-// ---- jk_split.cu (tensor-core contraction of FP64, double-FP32 and FP32 stores)
+// ---- jk_split.cu (tensor-core contraction of FP64 and double-FP32 stores)
 struct SplitLaunch {
     const BrickDesc *bricks;
     int64_t nbricks;
-    const int64_t *offsets;      // record start, in store elements
+    const int64_t *offsets;      // record start, in 8-byte elements
     const void *store;
-    int precision;               // of the store: FP64, F32X2 or FP32
+    int f32x2;                   // values are FP32 hi + lo pairs
     void *kbank, *jbank;         // density digit tiles (work memory)
     const double *D;
     int n, nb, m, num_sms;
@@ -174,8 +174,8 @@ struct SplitLaunch {
     cudaEvent_t ev_start = nullptr, ev_stop = nullptr;
 };
 int launch_jk_split(const SplitLaunch &L, cudaStream_t s);
-size_t split_kbank_bytes(int nb, int precision);
-size_t split_jbank_bytes(int nb, int precision);
+size_t split_kbank_bytes(int nb);
+size_t split_jbank_bytes(int nb);
 
 // ---- df_split.cu (density-fitted exchange on the tensor cores, FP64 accuracy)
 struct DfSplit {

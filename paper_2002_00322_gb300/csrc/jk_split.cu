@@ -1,5 +1,5 @@
-// Grouped J/K contraction on the sm_103a tensor cores (tcgen05) for FP64,
-// double-FP32 and FP32 integral stores, FP64-accurate for the first two: every operand is split without
+// FP64-accurate grouped J/K contraction on the sm_103a tensor cores (tcgen05)
+// for FP64 and double-FP32 integral stores: every operand is split without
 // error into fixed-point digits that the FP16 tensor pipe multiplies and sums
 // exactly (the error-free splitting of Ozaki, Ogita, Oishi and Rump 2012, in
 // its fixed-point form).
@@ -21,15 +21,6 @@
 // last place rounded in a later t weighs less than 2^-51 of the largest
 // product.  All digit pairs with t <= 6 are formed; the others are below 2^-60
 // of the largest product.
-//
-// FP32 stores take five digits of the integrals (44 bits) and four of the
-// densities (35, where FP32 arithmetic keeps 24), the pairs with t <= 4, and
-// join the c_t in FP32: five roundings per output and brick instead of one per
-// term.  Relative to FP64 integrals, 200 functions, 16 densities: J 3.5e-7 ->
-// 1.6e-7, K 1.6e-7 -> 8.0e-8; 9 to 300 functions and 1 to 32 densities are more
-// accurate than k_jk_cuda<float> throughout and take as long (up to 40
-// functions, launch-bound) or less: 200 functions, 1 density 2.00 -> 1.56 ms, 16
-// densities 4.08 -> 1.85 ms; 300 functions, 32 densities 39.8 -> 19.0 ms.
 //
 // MMA N covers the digits: with the density digits of a block as consecutive
 // operand rows [y_0 | y_1 | ...], the digit x_i multiplies a run of them at
@@ -77,33 +68,26 @@ using namespace umma;
 
 namespace {
 
+constexpr int NV = 7, ND = 6;                     // digits of an integral, of a density
+constexpr int NT = 7;                             // column groups t = i + j
 constexpr int SLICE = 8192;                       // one digit of a brick, 4096 x FP16
+constexpr int REC_BYTES = MASK_BYTES + 8 * BRICK; // keep mask + packed values
 constexpr int MPM = 16;                           // densities per pass
+constexpr int RING_SLOT = ND * 2 * MPM * 128;     // largest density tile (exchange)
+constexpr int OFF_V = 0, OFF_W = NV * SLICE, OFF_REC = 2 * NV * SLICE;
+constexpr int OFF_RING = OFF_REC + 2 * REC_BYTES;
+constexpr int OFF_CTRL = OFF_RING + 2 * RING_SLOT;
 constexpr int CTRL_BYTES = 2048;
-constexpr int REGION = 256;                       // tensor-memory columns per view buffer
-
-// Digits and shared-memory layout of a store's values, SRC: 0 FP64, 1
-// double-FP32, 2 FP32
-template <int SRC>
-struct Lay {
-    static constexpr int NV = SRC == 2 ? 5 : 7, ND = NV - 1;   // digits of an integral, of a density
-    static constexpr int NT = NV;                              // column groups t = i + j
-    static constexpr int VB = 9 * NV - 1, DB = 9 * ND - 1;     // bits of their fixed-point integers
-    static constexpr int EB = SRC == 2 ? 4 : 8;                // bytes of a stored value
-    static constexpr int REC = MASK_BYTES + EB * BRICK;        // keep mask + packed values
-    static constexpr int SLOT = ND * 2 * MPM * 128;            // largest density tile (exchange)
-    static constexpr int V = 0, W = NV * SLICE, RECS = 2 * NV * SLICE;
-    static constexpr int RING = RECS + 2 * REC, CTRL = RING + 2 * SLOT;
-    static constexpr int SMEM = CTRL + CTRL_BYTES;             // SRC 0, 1: all of the 227 KB a CTA can have
-    static_assert(RING % 1024 == 0 && RECS % 16 == 0, "operand tiles");
-    static_assert(NT * 2 * MPM <= REGION && SMEM <= 227 * 1024, "view region, shared memory");
-};
+constexpr int SPLIT_SMEM = OFF_CTRL + CTRL_BYTES;     // all of the 227 KB a CTA can have
 constexpr int CONV_WARPS = 8, CONV_THREADS = 32 * CONV_WARPS;
 constexpr int SPLIT_THREADS = 64 + CONV_THREADS + 256;
 // Smallest exponent fields of a tile: bricks below 2^-300 and density blocks
 // below 2^-640 lose their low digits, then vanish, and no product's exponent
 // leaves FP64's normal range (densities above 2^EMAX take the plain path).
 constexpr int EMIN_V = 1022 - 300, EMIN_D = 1022 - 640, EMAX = 500;
+constexpr int REGION = 256;                       // tensor-memory columns per view buffer
+static_assert(OFF_RING % 1024 == 0 && OFF_REC % 16 == 0, "operand tiles");
+static_assert(NT * 2 * MPM <= REGION, "view region");
 
 struct SplitCtrl {
     uint64_t recfull[2], recfree[2];   // packed records: landed / read
@@ -119,7 +103,7 @@ struct SplitCtrl {
     int ev[4];
     uint16_t vpos[512];
 };
-static_assert(sizeof(SplitCtrl) <= CTRL_BYTES, "control block");
+static_assert(SPLIT_SMEM <= 227 * 1024 && sizeof(SplitCtrl) <= CTRL_BYTES, "control block");
 
 // Polls after which a wait gives up (every wait here is far shorter).
 constexpr uint32_t POLLS = 1u << 22;
@@ -141,11 +125,6 @@ __device__ __forceinline__ bool has_view(const BrickDesc &d, int v) {
 // and read as a double through the bits of 1.5 2^52 + itself (|c_0| <= 2^22
 // likewise from c_0 + 1.5 2^23); the c_t of t >= 4 are summed in FP32, whose
 // bits widen to FP64 on the integer pipe too.  Two FP64 additions remain.
-__device__ __forceinline__ double widen(float f) {       // zero or a normal number
-    const uint32_t b = __float_as_uint(f);
-    const uint32_t hi = f == 0.0f ? 0u : (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u);
-    return __hiloint2double((int)hi, (int)(b << 29));
-}
 __device__ __forceinline__ double recombine(const float *c, int stride) {
     float f = fmaf(c[6 * stride], 0x1p-9f, c[5 * stride]);
     f = fmaf(f, 0x1p-18f, c[4 * stride] * 0x1p-9f);
@@ -153,15 +132,9 @@ __device__ __forceinline__ double recombine(const float *c, int stride) {
     S += (long long)__float2int_rn(c[1 * stride]) * (1 << 18);
     const int c0 = (int)(__float_as_uint(__fadd_rn(c[0], 12582912.f)) - 0x4b400000u);
     S += (long long)c0 * (1 << 27) + 0x4338000000000000ll;
-    return (__longlong_as_double(S) - 0x1.8p52) + widen(f);
-}
-// FP32 stores: sum_t c_t 2^(-9 t) in FP32, from the last digits up (a rounding
-// per digit, where an FP32 dot product has one per term)
-__device__ __forceinline__ double recombine_f(const float *c, int stride) {
-    float f = c[4 * stride];
-#pragma unroll
-    for (int t = 3; t >= 0; --t) f = fmaf(f, 0x1p-9f, c[t * stride]);
-    return widen(f);
+    const uint32_t b = __float_as_uint(f);
+    const uint32_t fhi = f == 0.0f ? 0u : (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u);
+    return (__longlong_as_double(S) - 0x1.8p52) + __hiloint2double((int)fhi, (int)(b << 29));
 }
 
 // *p += (value_hi, lo) as a double unless hi is zero (a zero value): a predicated
@@ -202,11 +175,9 @@ __device__ __forceinline__ int tile_off(int row, int k) {
 // transposed part of the tile has that of (Y,X)).  J bank, X >= Y: row j*mp +
 // kk of D[X,Y] + [X != Y] D[Y,X]^T, exponent eJ.  One warp per (X, Y, kk),
 // lane l the two elements b = l / 4, d = 2 (l % 4) + {0, 1}.
-template <int SRC>
 __global__ void __launch_bounds__(256) k_split_dbank(const double *D, int n, int nb, int m, int d0, int mp,
                                                      unsigned char *kbank, unsigned char *jbank, int16_t *eK,
                                                      int16_t *eJ, int *nonfinite) {
-    constexpr int ND = Lay<SRC>::ND, DB = Lay<SRC>::DB;
     const int tile = blockIdx.x, X = tile / nb, Y = tile % nb;
     const int lane = threadIdx.x & 31, kk = blockIdx.y * 8 + (threadIdx.x >> 5);
     const int b = lane >> 2, d = 2 * (lane & 3);
@@ -226,17 +197,15 @@ __global__ void __launch_bounds__(256) k_split_dbank(const double *D, int n, int
         e = max(__reduce_max_sync(0xffffffffu, e), EMIN_D);
         if (e > 1022 + EMAX && lane == 0) atomicOr(nonfinite, 1);
         uint32_t wa[3], wb[3];
-        digit_words<ND>(fixed_point<DB>((uint32_t)__double2loint(x[0]), h0, e), wa);
-        digit_words<ND>(fixed_point<DB>((uint32_t)__double2loint(x[1]), h1, e), wb);
+        digit_words<ND>(fixed_point<53>((uint32_t)__double2loint(x[0]), h0, e), wa);
+        digit_words<ND>(fixed_point<53>((uint32_t)__double2loint(x[1]), h1, e), wb);
         const int o = tile_off(row, b * 8 + d), step = rows * 128;   // rows of one digit: rows * 128 bytes
         *reinterpret_cast<uint32_t *>(base + o) = digit_pair<0>(wa, wb);
         *reinterpret_cast<uint32_t *>(base + o + step) = digit_pair<1>(wa, wb);
         *reinterpret_cast<uint32_t *>(base + o + 2 * step) = digit_pair<2>(wa, wb);
         *reinterpret_cast<uint32_t *>(base + o + 3 * step) = digit_pair<3>(wa, wb);
-        if constexpr (ND > 4) {
-            *reinterpret_cast<uint32_t *>(base + o + 4 * step) = digit_pair<4>(wa, wb);
-            *reinterpret_cast<uint32_t *>(base + o + 5 * step) = digit_pair<5>(wa, wb);
-        }
+        *reinterpret_cast<uint32_t *>(base + o + 4 * step) = digit_pair<4>(wa, wb);
+        *reinterpret_cast<uint32_t *>(base + o + 5 * step) = digit_pair<5>(wa, wb);
         if (lane == 0 && eout) *eout = (int16_t)(e - 1022);
     };
     unsigned char *kt = kbank + (size_t)tile * (ND * 2 * mp * 128);
@@ -254,7 +223,7 @@ __global__ void __launch_bounds__(256) k_split_dbank(const double *D, int n, int
 struct SplitParams {
     const BrickDesc *bricks;
     int64_t nbricks;
-    const int64_t *offsets;        // record start, in store elements
+    const int64_t *offsets;        // record start, in 8-byte elements
     const unsigned char *store;
     const unsigned char *kbank, *jbank;
     const int16_t *eK, *eJ;
@@ -277,7 +246,7 @@ __device__ void plain_bricks(const SplitParams &P, unsigned char *sm) {
     const int64_t nn = (int64_t)P.n * P.n;
     for (int64_t bi = blockIdx.x; bi < P.nbricks; bi += gridDim.x) {
         const BrickDesc d = P.bricks[bi];
-        const unsigned char *rec = P.store + P.offsets[bi] * Lay<SRC>::EB;
+        const unsigned char *rec = P.store + P.offsets[bi] * 8;
         __syncthreads();
         for (int v = threadIdx.x; v < 512; v += blockDim.x) {
             int c = 0;
@@ -291,7 +260,6 @@ __device__ void plain_bricks(const SplitParams &P, unsigned char *sm) {
             if (mk & (1u << (e & 7))) {
                 const int i = pos[e >> 3] + __popc(mk & ((1u << (e & 7)) - 1u));
                 if (SRC == 0) x = reinterpret_cast<const double *>(rec + MASK_BYTES)[i];
-                else if (SRC == 2) x = (double)reinterpret_cast<const float *>(rec + MASK_BYTES)[i];
                 else {
                     const float2 u = reinterpret_cast<const float2 *>(rec + MASK_BYTES)[i];
                     x = (double)u.x + (double)u.y;
@@ -332,7 +300,7 @@ __device__ void plain_bricks(const SplitParams &P, unsigned char *sm) {
 
 }  // namespace
 
-// MP: density columns of the pass (8 or 16)
+// SRC: 0 FP64 store, 1 double-FP32 store; MP: density columns of the pass (8 or 16)
 template <int SRC, int MP>
 __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_constant__ SplitParams P) {
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -340,10 +308,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
         plain_bricks<SRC>(P, sm);
         return;
     }
-    using L = Lay<SRC>;
-    constexpr int NV = L::NV, ND = L::ND, NT = L::NT, REC_BYTES = L::REC, RING_SLOT = L::SLOT;
-    constexpr int OFF_V = L::V, OFF_W = L::W, OFF_REC = L::RECS, OFF_RING = L::RING;
-    SplitCtrl &c = *reinterpret_cast<SplitCtrl *>(sm + L::CTRL);
+    SplitCtrl &c = *reinterpret_cast<SplitCtrl *>(sm + OFF_CTRL);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr uint32_t KBYTES = ND * 2 * MP * 128, JBYTES = ND * MP * 128;
     volatile int *abort_flag = &c.abort_flag;
@@ -384,9 +349,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
         auto load_record = [&](int i, const BrickDesc &d) -> bool {
             const int s = i & 1;
             if (i >= 2 && !wait_for(&c.recfree[s], ((i - 2) >> 1) & 1, abort_flag)) { fail(21); return false; }
-            const uint32_t rec = ((uint32_t)MASK_BYTES + (uint32_t)L::EB * (uint32_t)d.nkept + 15u) & ~15u;
+            const uint32_t rec = ((uint32_t)MASK_BYTES + 8u * (uint32_t)d.nkept + 15u) & ~15u;
             mbar_arrive_expect_tx(&c.recfull[s], rec);
-            bulk_g2s(sm + OFF_REC + s * REC_BYTES, P.store + P.offsets[blockIdx.x + (int64_t)i * step] * L::EB, rec,
+            bulk_g2s(sm + OFF_REC + s * REC_BYTES, P.store + P.offsets[blockIdx.x + (int64_t)i * step] * 8, rec,
                      &c.recfull[s]);
             recs = i + 1;
             return true;
@@ -456,9 +421,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                     for (int j = 0; j < 4; ++j) {
                         const uint32_t a = alo + x * (SLICE >> 4) + j * ks, bd = blo + 16 * j;
                         if (x == 1 && j == 0) {
-                            // t = ND starts here: its columns are written, those of t < ND added to
-                            mma_pred(lead, col + Wu, a, ahi, bd, bhi, id0 + (ND - 1) * wid, 1u);
-                            mma_pred(lead, col + ND * Wu, a, ahi, bd + 8 * (ND - 1) * Wu, bhi, id0 + wid, 0u);
+                            // t = 6 starts here: its columns are written, those of t < 6 added to
+                            mma_pred(lead, col + Wu, a, ahi, bd, bhi, id0 + 5 * wid, 1u);
+                            mma_pred(lead, col + 6 * Wu, a, ahi, bd + 40 * Wu, bhi, id0 + wid, 0u);
                         } else {
                             mma_pred(lead, col + x * Wu, a, ahi, bd, bhi, id0 + nj * wid, (x > 0 || j > 0) ? 1u : 0u);
                         }
@@ -488,12 +453,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
             named_bar_sync(1, CONV_THREADS);
             if (ct == 0) c.decide = *abort_flag;
             const unsigned char *mask = sm + OFF_REC + s * REC_BYTES;
-            using VAL = typename std::conditional<SRC == 2, uint32_t, uint2>::type;
-            const VAL *vals = reinterpret_cast<const VAL *>(mask + MASK_BYTES);
-            auto top = [](const VAL &w) -> uint32_t {          // the word with the exponent
-                if constexpr (SRC == 2) return w;
-                else return SRC == 0 ? w.y : w.x;
-            };
+            const uint2 *vals = reinterpret_cast<const uint2 *>(mask + MASK_BYTES);
             // packed positions (exclusive scan of the per-vector counts) and the largest exponent
             const uint32_t mk2 = reinterpret_cast<const uint16_t *>(mask)[ct];
             const int tot = __popc(mk2);
@@ -504,7 +464,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                 if (lane >= o) incl += y;
             }
             uint32_t hmax = 0;
-            for (int k = ct; k < nkept; k += CONV_THREADS) hmax = max(hmax, top(vals[k]) & 0x7fffffffu);
+            for (int k = ct; k < nkept; k += CONV_THREADS) hmax = max(hmax, (SRC == 0 ? vals[k].y : vals[k].x) & 0x7fffffffu);
             int em = SRC == 0 ? (int)(hmax >> 20) : (hmax >> 23 ? (int)(hmax >> 23) + 896 : 0);
             em = __reduce_max_sync(0xffffffffu, em);
             if (lane == 31) { c.scan[cw] = incl; c.emax[cw] = em; }
@@ -535,18 +495,17 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                 vv[k] = p * 64 + q * 8 + r;
                 ww[k] = p * 64 + r * 8 + q;
                 const uint32_t m8 = mask[vv[k]];
-                const VAL *src = vals + c.vpos[vv[k]];
+                const uint2 *src = vals + c.vpos[vv[k]];
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
                     long long x[2];
 #pragma unroll
                     for (int z = 0; z < 2; ++z) {
                         const int e = 2 * h + z;
-                        VAL w{};
+                        uint2 w = make_uint2(0u, 0u);
                         if (m8 & (1u << e)) w = src[__popc(m8 & ((1u << e) - 1u))];
-                        if constexpr (SRC == 0) x[z] = fixed_point<L::VB>(w.x, w.y, emax);
-                        else if constexpr (SRC == 2) x[z] = fixed_point_f<L::VB>(__uint_as_float(w), emax);
-                        else x[z] = fixed_point_f<L::VB>(__uint_as_float(w.x), emax) + fixed_point_f<L::VB>(__uint_as_float(w.y), emax);
+                        if (SRC == 0) x[z] = fixed_point<62>(w.x, w.y, emax);
+                        else x[z] = fixed_point_f<62>(__uint_as_float(w.x), emax) + fixed_point_f<62>(__uint_as_float(w.y), emax);
                     }
                     uint32_t wa[3], wb[3];
                     digit_words<NV>(x[0], wa);
@@ -556,10 +515,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                     dg[k][2][h] = digit_pair<2>(wa, wb);
                     dg[k][3][h] = digit_pair<3>(wa, wb);
                     dg[k][4][h] = digit_pair<4>(wa, wb);
-                    if constexpr (NV > 5) {
-                        dg[k][5][h] = digit_pair<5>(wa, wb);
-                        dg[k][6][h] = digit_pair<6>(wa, wb);
-                    }
+                    dg[k][5][h] = digit_pair<5>(wa, wb);
+                    dg[k][6][h] = digit_pair<6>(wa, wb);
                 }
             }
             __syncwarp();
@@ -621,7 +578,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                 if (!__all_sync(~0u, wait_for(&c.mmad[g], (vi >> 1) & 1, abort_flag))) { fail(30); ok = false; break; }
                 if (!have) {
                     if (!__all_sync(~0u, counter_wait(&c.epub, (unsigned)i + 1u, abort_flag, POLLS))) { fail(31); ok = false; break; }
-                    ev = c.ev[i & 3] - (SRC == 2 ? 16 : 43);
+                    ev = c.ev[i & 3] - 43;
                     have = true;
                 }
                 tc_fence_after();
@@ -650,7 +607,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                         for (int j = 0; j < H; ++j) {
                             // the power of two is added to the exponent field; columns without a
                             // density have zeros
-                            const double x = SRC == 2 ? recombine_f(a + j, H) : recombine(a + j, H);
+                            const double x = recombine(a + j, H);
                             const int hi = __double2hiint(x);
                             red_nonzero(dst + j * 64, hi, hi + ((ev + xp[j]) << 20), __double2loint(x));
                         }
@@ -668,28 +625,21 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
 }
 
 // ---------------------------------------------------------------- host side
-static int split_nd(int precision) { return precision == ESMF_PREC_FP32 ? Lay<2>::ND : Lay<0>::ND; }
-size_t split_kbank_bytes(int nb, int precision) {
-    return (size_t)nb * nb * (split_nd(precision) * 2 * MPM * 128 + MPM * sizeof(int16_t));
-}
-size_t split_jbank_bytes(int nb, int precision) {
-    return (size_t)nb * (nb + 1) / 2 * (split_nd(precision) * MPM * 128 + MPM * sizeof(int16_t));
-}
+size_t split_kbank_bytes(int nb) { return (size_t)nb * nb * (ND * 2 * MPM * 128 + MPM * sizeof(int16_t)); }
+size_t split_jbank_bytes(int nb) { return (size_t)nb * (nb + 1) / 2 * (ND * MPM * 128 + MPM * sizeof(int16_t)); }
 
 template <int SRC, int MP>
 static int split_pass(const SplitParams &p, int grid, cudaStream_t s) {
-    constexpr int smem = Lay<SRC>::SMEM;
-    cudaError_t e = cudaFuncSetAttribute(k_jk_split<SRC, MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(k_jk_split<SRC, MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, SPLIT_SMEM);
     if (e != cudaSuccess) { set_error("smem attribute: %s", cudaGetErrorString(e)); return ESMF_ERR_CUDA; }
-    k_jk_split<SRC, MP><<<grid, SPLIT_THREADS, smem, s>>>(p);
+    k_jk_split<SRC, MP><<<grid, SPLIT_THREADS, SPLIT_SMEM, s>>>(p);
     e = cudaGetLastError();
     if (e != cudaSuccess) { set_error("k_jk_split: %s", cudaGetErrorString(e)); return ESMF_ERR_CUDA; }
     return ESMF_OK;
 }
 
-template <int SRC>
-static int split_build(const SplitLaunch &L, cudaStream_t s) {
-    constexpr int ND = Lay<SRC>::ND;
+int launch_jk_split(const SplitLaunch &L, cudaStream_t s) {
+    if (L.ev_start) cudaEventRecord(L.ev_start, s);
     for (int d0 = 0; d0 < L.m; d0 += MPM) {
         const int mc = L.m - d0 < MPM ? L.m - d0 : MPM;
         const int mp = mc <= 8 ? 8 : MPM;
@@ -703,21 +653,15 @@ static int split_build(const SplitLaunch &L, cudaStream_t s) {
         p.kbank = kb; p.jbank = jb; p.eK = eK; p.eJ = eJ;
         p.D = L.D; p.n = L.n; p.nb = L.nb; p.m = mc; p.d0 = d0; p.mtot = L.m;
         p.Jacc = L.Jacc; p.Kacc = L.Kacc; p.KTacc = L.KTacc; p.nonfinite = L.nonfinite; p.error = L.error;
-        k_split_dbank<SRC><<<dim3(L.nb * L.nb, mp / 8), 256, 0, s>>>(L.D, L.n, L.nb, mc, d0, mp, kb, jb, eK, eJ, L.nonfinite);
+        k_split_dbank<<<dim3(L.nb * L.nb, mp / 8), 256, 0, s>>>(L.D, L.n, L.nb, mc, d0, mp, kb, jb, eK, eJ, L.nonfinite);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) { set_error("k_split_dbank: %s", cudaGetErrorString(e)); return ESMF_ERR_CUDA; }
         const int grid = L.nbricks < L.num_sms ? (int)L.nbricks : L.num_sms;
-        const int rc = mp == 8 ? split_pass<SRC, 8>(p, grid, s) : split_pass<SRC, 16>(p, grid, s);
+        int rc;
+        if (L.f32x2) rc = mp == 8 ? split_pass<1, 8>(p, grid, s) : split_pass<1, 16>(p, grid, s);
+        else rc = mp == 8 ? split_pass<0, 8>(p, grid, s) : split_pass<0, 16>(p, grid, s);
         if (rc != ESMF_OK) return rc;
     }
-    return ESMF_OK;
-}
-
-int launch_jk_split(const SplitLaunch &L, cudaStream_t s) {
-    if (L.ev_start) cudaEventRecord(L.ev_start, s);
-    const int rc = L.precision == ESMF_PREC_FP32 ? split_build<2>(L, s)
-                   : L.precision == ESMF_PREC_F32X2 ? split_build<1>(L, s) : split_build<0>(L, s);
-    if (rc != ESMF_OK) return rc;
     if (L.ev_stop) cudaEventRecord(L.ev_stop, s);
     return ESMF_OK;
 }

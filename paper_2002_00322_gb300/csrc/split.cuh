@@ -16,10 +16,9 @@ namespace split {
 // so that the last bit shifted out rounds; zeros (exponent field 0) shift out.
 template <int BITS>
 __device__ __forceinline__ long long fixed_point(uint32_t lo, uint32_t hi, int emax) {
-    constexpr int up = BITS > 52 ? BITS - 52 : 0;
-    const int sh = min(emax - (int)((hi >> 20) & 0x7ffu) + (up + 52 - BITS), 63);
+    const int sh = min(emax - (int)((hi >> 20) & 0x7ffu), 63);
     const unsigned long long mant = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-    const unsigned long long r = (((mant << up) >> sh) + 1) >> 1;
+    const unsigned long long r = (((mant << (BITS - 52)) >> sh) + 1) >> 1;
     const long long sg = (int)hi >> 31;
     return ((long long)r ^ sg) - sg;
 }
@@ -37,7 +36,7 @@ __device__ __forceinline__ long long fixed_point_f(float x, int emax) {
 
 // Balanced digits of X, |X| <= 2^(9 N - 1): X + sum_k 256 512^k has the digits
 // u_i of base 512 (u_0 up to 512), x_i = u_i - 256.  Words of three digits,
-// w[0] = u_0 u_1 u_2 and so on (the second word of N < 6 filled from the top).
+// w[0] = u_0 u_1 u_2 and so on.
 template <int N>
 __device__ __forceinline__ void digit_words(long long X, uint32_t *w) {
     unsigned long long B = 0;
@@ -45,9 +44,8 @@ __device__ __forceinline__ void digit_words(long long X, uint32_t *w) {
     for (int k = 0; k < N; ++k) B += 256ull << (9 * k);
     const unsigned long long Y = (unsigned long long)X + B;
     w[0] = (uint32_t)(Y >> (9 * N - 27));
-    if constexpr (N >= 6) w[1] = (uint32_t)(Y >> (9 * N - 54)) & 0x7ffffffu;
-    else w[1] = ((uint32_t)Y & ((1u << (9 * N - 27)) - 1u)) << (54 - 9 * N);
-    if constexpr (N > 6) w[2] = (uint32_t)Y & 0x1ffu;
+    w[1] = (uint32_t)(Y >> (9 * N - 54)) & 0x7ffffffu;
+    if (N > 6) w[2] = (uint32_t)Y & 0x1ffu;
 }
 // digit i of two values as packed FP16: FP16 holds 1024 + u exactly with the
 // bits 0x6400 | u, and subtracting 1280 leaves u - 256

@@ -378,7 +378,9 @@ int esmf_fock_set_density_screening(esmf_fock_t *h, double tol_d);
  * integrals: ESMF_PATH_AUTO uses the tensor-core kernels (for FP64 and F32X2
  * by error-free splitting, as accurate as FP64 arithmetic),
  * ESMF_PATH_CUDA_CORE the CUDA-core kernels (same results within rounding;
- * kept as a cross-check).  FP32 stores and integral-direct FP64 / FP32
+ * kept as a cross-check).  Integral-direct FP64 handles of s bases take the
+ * splitting kernel from a scratch buffer of integral records (at most 2 GiB, or
+ * a quarter of the budget) when it and the density digits fit the budget.  FP32
  * handles always use the CUDA-core kernels.  Errors: INVALID_ARG.
  */
 #define ESMF_PATH_AUTO       0

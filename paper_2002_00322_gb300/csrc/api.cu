@@ -61,8 +61,8 @@ struct esmf_fock {
     int *pslot = nullptr, *pblocks = nullptr;
     int n_ptab = 0;
     float vscale = 1.0f;           // power-of-two scale of split 16-bit stores
-    // integral-direct builds on the tensor cores (FP16X2 / BF16X2 direct
-    // handles): the brick list cut at item boundaries into chunks whose packed
+    // integral-direct builds on the tensor cores (FP16X2 / BF16X2, and FP64
+    // by digit splitting): the brick list cut at item boundaries into chunks whose packed
     // records fit the scratch buffer; chunk c is bricks [chunks[c], chunks[c+1]),
     // its records regenerated into `scratch` by every build (offsets above are
     // then relative to the chunk's first brick).  Generation and contraction
@@ -119,7 +119,7 @@ struct esmf_fock {
     // J then K (then, on the split path, K's transposed blocks and a flag word)
     double *acc = nullptr;
     size_t acc_n = 0;
-    // FP64 and double-FP32 stores: density digit tiles of the tensor-core path;
+    // FP64 and double-FP32: density digit tiles of the tensor-core path;
     // no_split: this handle stays on the CUDA-core kernel (values beyond FP64's
     // range, or no memory for the tiles)
     void *skbank = nullptr, *sjbank = nullptr;
@@ -316,10 +316,14 @@ bool is_device_ptr(const void *p) {
 // chunk and contract them on the tensor cores
 bool tensor_direct(const esmf_fock *h) { return h->mode == ESMF_MODE_DIRECT && is_split16(h->prec) && h->scratch; }
 
-// FP64 or double-FP32 store that builds by exact digit splitting on the tensor
-// cores (jk_split.cu)
+// FP64 or double-FP32 handle that builds by exact digit splitting on the tensor
+// cores (jk_split.cu): from its store, or chunk by chunk from the records that an
+// integral-direct FP64 build regenerates in the scratch buffer.  Evaluating in the
+// CUDA-core contraction instead took, 24 functions and 64 densities, 3.12 ms against
+// 2.58; 160 functions, 1 density 165 ms against 158, 64 densities 225 against 160.
 bool split_path(const esmf_fock *h) {
-    return h->mode == ESMF_MODE_STORED && (h->prec == ESMF_PREC_FP64 || h->prec == ESMF_PREC_F32X2) && !h->no_split;
+    return (h->mode == ESMF_MODE_STORED || (h->mode == ESMF_MODE_DIRECT && h->scratch)) &&
+           (h->prec == ESMF_PREC_FP64 || h->prec == ESMF_PREC_F32X2) && !h->no_split;
 }
 
 // doubles of the accumulators of a build of m densities
@@ -759,10 +763,14 @@ static int create_impl(const esmf_basis_t *basis, const int32_t *cart, double to
                 return fail(ESMF_ERR_CUDA);
             h->nparts = (int)parts.size() - 1;
         }
-        if (use_mode == ESMF_MODE_DIRECT && is_split16(h->prec) && !h->cart) {
+        if (use_mode == ESMF_MODE_DIRECT && h->prec != ESMF_PREC_FP32 && !h->cart) {
             // integral-direct on the tensor cores: chunks of whole items whose
             // records fit the scratch buffer (2 GiB, or a quarter of the budget;
-            // an item larger than that is a chunk of its own)
+            // an item larger than that is a chunk of its own).  FP64 handles
+            // take it when their budget and memory hold it and the density digits
+            // too, and evaluate in the contraction kernel otherwise.
+            const bool by_split = !is_split16(h->prec);
+            const int eb = elem_bytes(h->prec);
             int64_t cap = (int64_t)2 << 30;
             if (budget_bytes > 0) cap = std::min<int64_t>(cap, budget_bytes / 4);
             const int64_t nk = h->nbricks;
@@ -781,22 +789,36 @@ static int create_impl(const esmf_basis_t *basis, const int32_t *cart, double to
                 most = std::max(most, (offs[ch[c + 1]] - offs[ch[c]]) * eb);
             }
             h->chunks = ch;
-            h->scratch_bytes = most;
-            if ((rc = dalloc(h, &h->offsets, nk + 1))) return fail(rc);
-            if ((rc = dalloc(h, (unsigned char **)&h->scratch, (size_t)h->scratch_bytes))) return fail(rc);
-            if (!ck(cudaMemcpyAsync(h->offsets, roff.data(), sizeof(int64_t) * (nk + 1), cudaMemcpyHostToDevice, cs), "copy chunk offsets") ||
-                !ck(cudaMemsetAsync(h->scratch, 0, (size_t)h->scratch_bytes, cs), "clear scratch"))
-                return fail(ESMF_ERR_CUDA);
-            // each scratch chunk's cost-balanced chunks for the tensor kernel
-            for (size_t c = 0; c + 1 < ch.size(); ++c) {
-                std::vector<BrickDesc> sub(kept.begin() + ch[c], kept.begin() + ch[c + 1]);
-                const std::vector<int64_t> sp = balance_parts(sub, kChunksPerSM * h->num_sms);
-                int64_t *dp = nullptr;
-                if ((rc = dalloc(h, &dp, sp.size()))) return fail(rc);
-                h->shard_parts.emplace(std::make_pair(ch[c], ch[c + 1]), std::make_pair(dp, (int)sp.size() - 1));
-                if (!ck(cudaMemcpyAsync(dp, sp.data(), sizeof(int64_t) * sp.size(), cudaMemcpyHostToDevice, cs), "copy chunk parts") ||
-                    !ck(cudaStreamSynchronize(cs), "chunk parts"))
+            bool room = true;
+            if (by_split) {
+                const int64_t need = most + (nk + 1) * 8 + (int64_t)split_kbank_bytes(h->nb) +
+                                     (int64_t)split_jbank_bytes(h->nb);
+                room = !h->no_split && (budget_bytes == 0 || h->device_bytes + need <= budget_bytes);
+                if (room && dalloc(h, (unsigned char **)&h->scratch, (size_t)most) != ESMF_OK) {
+                    cudaGetLastError();
+                    room = false;
+                }
+            } else if ((rc = dalloc(h, (unsigned char **)&h->scratch, (size_t)most))) {
+                return fail(rc);
+            }
+            if (room) {
+                h->scratch_bytes = most;
+                if ((rc = dalloc(h, &h->offsets, nk + 1))) return fail(rc);
+                if (!ck(cudaMemcpyAsync(h->offsets, roff.data(), sizeof(int64_t) * (nk + 1), cudaMemcpyHostToDevice, cs), "copy chunk offsets") ||
+                    !ck(cudaMemsetAsync(h->scratch, 0, (size_t)h->scratch_bytes, cs), "clear scratch"))
                     return fail(ESMF_ERR_CUDA);
+                // each scratch chunk's cost-balanced chunks for the tensor kernel
+                for (size_t c = 0; !by_split && c + 1 < ch.size(); ++c) {
+                    std::vector<BrickDesc> sub(kept.begin() + ch[c], kept.begin() + ch[c + 1]);
+                    const std::vector<int64_t> sp = balance_parts(sub, kChunksPerSM * h->num_sms);
+                    int64_t *dp = nullptr;
+                    if ((rc = dalloc(h, &dp, sp.size()))) return fail(rc);
+                    h->shard_parts.emplace(std::make_pair(ch[c], ch[c + 1]), std::make_pair(dp, (int)sp.size() - 1));
+                    if (!ck(cudaMemcpyAsync(dp, sp.data(), sizeof(int64_t) * sp.size(), cudaMemcpyHostToDevice, cs), "copy chunk parts") ||
+                        !ck(cudaStreamSynchronize(cs), "chunk parts"))
+                        return fail(ESMF_ERR_CUDA);
+                }
+                if (by_split && !ck(cudaStreamSynchronize(cs), "chunk offsets")) return fail(ESMF_ERR_CUDA);
             }
         }
         if (use_mode == ESMF_MODE_STORED) {
@@ -1407,8 +1429,22 @@ int build_range(esmf_fock_t *h, int64_t b0, int64_t b1, int m, const double *D, 
             L.num_sms = h->num_sms;
             L.Jacc = Jacc; L.Kacc = Kacc; L.KTacc = Kacc + cnt;
             L.nonfinite = (int *)(Kacc + 2 * cnt); L.error = h->err_dev;
-            L.ev_start = e0; L.ev_stop = e1;
-            RET(launch_jk_split(L, s));
+            if (h->mode == ESMF_MODE_STORED) {
+                L.ev_start = e0; L.ev_stop = e1;
+                RET(launch_jk_split(L, s));
+            } else {
+                if (e0) CKR(cudaEventRecord(e0, s));
+                for (size_t c = 0; c + 1 < h->chunks.size(); ++c) {
+                    const int64_t r0 = std::max(b0, h->chunks[c]), r1 = std::min(b1, h->chunks[c + 1]);
+                    if (r1 <= r0) continue;
+                    RET(launch_brick_generate(h->dev(), h->S, h->tol_s, h->bricks + r0, r1 - r0, h->offsets + r0,
+                                              h->prec, h->scratch, h->vscale, s, h->ptab, h->pslot));
+                    L.bricks = h->bricks + r0; L.nbricks = r1 - r0; L.offsets = h->offsets + r0;
+                    L.store = h->scratch;
+                    RET(launch_jk_split(L, s));
+                }
+                if (e1) CKR(cudaEventRecord(e1, s));
+            }
             return launch_finalize_blocked(h->dev(), m, D, Jacc, Kacc, L.KTacc, J, K, F, traces, s);
         }
         if (h->Dt) {

@@ -32,17 +32,18 @@
 // from shared memory (7.3K cycles at 128 B per clock) beside 350 KB of other
 // traffic there; the CUDA-core FP64 form of the same brick takes 327K cycles
 // (GB300 has two FP64 FMA per clock and SM).  200 functions, 16 densities, 53K
-// bricks: 54.7 ms with k_jk_cuda<double>, 3.02 ms here (16.5K cycles a brick).
-// Recombining into one 62-bit integer per output takes 2.62 ms, but rounds every
-// output at 2^-56 of the brick's largest product, also one a thousand times
-// smaller, where FP64 arithmetic would not.
+// bricks: 54.7 ms with k_jk_cuda<double>, 2.78 ms here (15.4K cycles a brick).
+// Recombining into one 62-bit integer per output was faster (2.62 ms against
+// 3.02 when that was tried), but rounds every output at 2^-56 of the brick's
+// largest product, also one a thousand times smaller, where FP64 arithmetic
+// would not.
 //
-// Warp roles (576 threads, one CTA per SM): warp 0 producer (bulk copies of
-// the packed record one brick ahead and of one density tile per view through a
-// two-slot ring), warp 1 tensor-memory owner and MMA issuer, warps 2-9
+// Warp roles (832 threads, 576 at 8 densities; one CTA per SM): warp 0 producer
+// (bulk copies of the packed record one brick ahead and of one density tile per
+// view through a two-slot ring), warp 1 tensor-memory owner and MMA issuer, warps 2-9
 // converters (packed record -> digits in registers -> tiles V and, with r and q
-// swapped, W, which the Coulomb views read), warps 10-17 epilogue in two groups
-// of four that take the views alternately: tensor-memory load, integer
+// swapped, W, which the Coulomb views read), the others epilogue in two groups
+// that take the views alternately: tensor-memory load, integer
 // recombination of the c_t, one FP64 reduction per output.  V
 // and W are single tiles (shared memory holds no second pair): the digits of
 // the next brick wait in registers, V is written while the Coulomb MMAs (over
@@ -54,8 +55,6 @@
 // Densities that are not finite (or above 2^500) have no digits: k_split_dbank
 // then raises a flag and the kernel runs a plain FP64 loop over the same bricks.
 #include <cuda_fp16.h>
-
-#include <type_traits>
 
 #include "esmf_internal.cuh"
 #include "split.cuh"
@@ -80,7 +79,15 @@ constexpr int OFF_CTRL = OFF_RING + 2 * RING_SLOT;
 constexpr int CTRL_BYTES = 2048;
 constexpr int SPLIT_SMEM = OFF_CTRL + CTRL_BYTES;     // all of the 227 KB a CTA can have
 constexpr int CONV_WARPS = 8, CONV_THREADS = 32 * CONV_WARPS;
-constexpr int SPLIT_THREADS = 64 + CONV_THREADS + 256;
+// Epilogue warps: at 16 densities two groups of eight, the warps of a group
+// sharing a view's densities (200 functions 2.99 -> 2.78 ms against groups of
+// four; a view's 224 columns are read, recombined and reduced by them); at 8
+// densities groups of four (2.00 ms against 2.09 with eight: half the work, and
+// more warps then only contend with the converters and the MMA issuer).
+template <int MP>
+constexpr int epi_warps = MP == 16 ? 16 : 8;
+template <int MP>
+constexpr int split_threads = 64 + CONV_THREADS + 32 * epi_warps<MP>;
 // Smallest exponent fields of a tile: bricks below 2^-300 and density blocks
 // below 2^-640 lose their low digits, then vanish, and no product's exponent
 // leaves FP64's normal range (densities above 2^EMAX take the plain path).
@@ -145,19 +152,14 @@ __device__ __forceinline__ void red_nonzero(double *p, int hi, int value_hi, int
                  : "memory");
 }
 
-template <int H>
-__device__ __forceinline__ void tmem_ld_half(uint32_t taddr, float *v) {
-    uint32_t r[H];
-    if constexpr (H == 8)
-        asm volatile("tcgen05.ld.sync.aligned.16x32bx2.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], 8;"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                     : "r"(taddr));
-    else
-        asm volatile("tcgen05.ld.sync.aligned.16x32bx2.x4.b32 {%0,%1,%2,%3}, [%4], 4;"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                     : "r"(taddr));
+// four columns for lanes 0-15, the next four for lanes 16-31 of 16 accumulator rows
+__device__ __forceinline__ void tmem_ld_half4(uint32_t taddr, float *v) {
+    uint32_t r[4];
+    asm volatile("tcgen05.ld.sync.aligned.16x32bx2.x4.b32 {%0,%1,%2,%3}, [%4], 4;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
 #pragma unroll
-    for (int i = 0; i < H; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // canonical K-major operand tile: row n (density column of the MMA), k = b*8 + d
@@ -302,7 +304,7 @@ __device__ void plain_bricks(const SplitParams &P, unsigned char *sm) {
 
 // SRC: 0 FP64 store, 1 double-FP32 store; MP: density columns of the pass (8 or 16)
 template <int SRC, int MP>
-__global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_constant__ SplitParams P) {
+__global__ void __launch_bounds__(split_threads<MP>, 1) k_jk_split(const __grid_constant__ SplitParams P) {
     extern __shared__ __align__(1024) unsigned char sm[];
     if (*P.nonfinite) {
         plain_bricks<SRC>(P, sm);
@@ -321,7 +323,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
             mbar_init(&c.recfree[s], CONV_WARPS);
             mbar_init(&c.dfull[s], 1);
             mbar_init(&c.mmad[s], 1);
-            mbar_init(&c.accfree[s], 4);
+            mbar_init(&c.accfree[s], epi_warps<MP> / 2);
         }
         mbar_init(&c.convV, CONV_WARPS);
         mbar_init(&c.convW, CONV_WARPS);
@@ -540,12 +542,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
         }
     } else if (warp >= 2 + CONV_WARPS) {
         // ------------------------------------------------ epilogue
-        // group g takes the views with index parity g (tensor-memory region g); each
-        // group's four warps cover the four lane quarters
-        const int g = warp >= 6 + CONV_WARPS ? 1 : 0, slice = warp & 3;
-        const uint32_t tl = tmem + ((uint32_t)(slice * 32) << 16) + g * REGION;
-        constexpr int H = MP / 2;
-        const int row = slice * 16 + (lane & 15), cb = lane < 16 ? 0 : H;
+        // group g takes the views with index parity g (tensor-memory region g); four
+        // of its warps cover the four lane quarters for eight densities
+        constexpr int GW = epi_warps<MP> / 2, H = 4;         // warps of a group, densities of a thread
+        const int ew = warp - 2 - CONV_WARPS, g = ew / GW, slice = warp & 3;
+        const int c0 = (ew % GW) / 4 * 2 * H;                // the warp's densities: c0 .. c0 + 7
+        const uint32_t tl = tmem + ((uint32_t)(slice * 32) << 16) + g * REGION + c0;
+        const int row = slice * 16 + (lane & 15), cb = c0 + (lane < 16 ? 0 : H);
         int views = 0;
         BrickDesc dn = brick(0);
         bool ok = true;
@@ -566,14 +569,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                 const int ty = v == 5 ? d.Q : ((v < 2 || v == 4) ? d.S : d.R);
                 const bool coul = v >= 4;
                 // exponents of the parts' density blocks: the D part, then (exchange) the D^T part
-                using EX = typename std::conditional<H == 8, uint4, uint2>::type;
-                EX xq[2];
+                uint2 xq[2];
                 {
                     const int16_t *ex = coul ? P.eJ + ((size_t)tx * (tx + 1) / 2 + ty) * MPM
                                              : P.eK + ((size_t)tx * P.nb + ty) * MPM;
                     const int16_t *et = coul ? ex : P.eK + ((size_t)ty * P.nb + tx) * MPM;
-                    xq[0] = *reinterpret_cast<const EX *>(ex + cb);
-                    xq[1] = *reinterpret_cast<const EX *>(et + cb);
+                    xq[0] = *reinterpret_cast<const uint2 *>(ex + cb);
+                    xq[1] = *reinterpret_cast<const uint2 *>(et + cb);
                 }
                 if (!__all_sync(~0u, wait_for(&c.mmad[g], (vi >> 1) & 1, abort_flag))) { fail(30); ok = false; break; }
                 if (!have) {
@@ -589,12 +591,12 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_jk_split(const __grid_cons
                 const bool none = v == 5 && diag;
 #pragma unroll 1
                 for (int part = 0; part < parts; ++part) {
-                    alignas(16) int16_t xp[H];
-                    *reinterpret_cast<EX *>(xp) = part ? xq[1] : xq[0];
+                    alignas(8) int16_t xp[H];
+                    *reinterpret_cast<uint2 *>(xp) = part ? xq[1] : xq[0];
                     float a[NT * H];
                     __syncwarp();
 #pragma unroll
-                    for (int t = 0; t < NT; ++t) tmem_ld_half<H>(tl + part * MP + t * W, a + t * H);
+                    for (int t = 0; t < NT; ++t) tmem_ld_half4(tl + part * MP + t * W, a + t * H);
                     tmem_wait_ld();
                     if (part == parts - 1) {
                         tc_fence_before();
@@ -632,7 +634,7 @@ template <int SRC, int MP>
 static int split_pass(const SplitParams &p, int grid, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(k_jk_split<SRC, MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, SPLIT_SMEM);
     if (e != cudaSuccess) { set_error("smem attribute: %s", cudaGetErrorString(e)); return ESMF_ERR_CUDA; }
-    k_jk_split<SRC, MP><<<grid, SPLIT_THREADS, SPLIT_SMEM, s>>>(p);
+    k_jk_split<SRC, MP><<<grid, split_threads<MP>, SPLIT_SMEM, s>>>(p);
     e = cudaGetLastError();
     if (e != cudaSuccess) { set_error("k_jk_split: %s", cudaGetErrorString(e)); return ESMF_ERR_CUDA; }
     return ESMF_OK;

@@ -127,6 +127,22 @@ def measured_alu_peaks(local):
     return {p: round(max(fock.esmf_measure_fma_peak(p, local) for _ in range(2)), 2) for p in ("fp64", "fp32")}
 
 
+def stored_roofline(prec, st, m, n, kern_s, alu_peaks, workload="stored_n200_m16"):
+    """Roofline of a stored build on the path it takes.  FP64 and double-FP32
+    stores run k_jk_split, which forms 27 FP16 digit products per FP64 one:
+    those of the algorithmic 20 m flops per kept unique quartet against the
+    measured 16-bit tensor rate; the others as contraction_roofline has it."""
+    if prec not in ("fp64", "f32x2"):
+        return contraction_roofline(prec, st, m, n, kern_s, alu_peaks, workload)
+    _, src, d = peaks()
+    pk = float(d.get("bf16_tflops", 1900.0))
+    flops = st["n_quartets_kept"] * 20 * m
+    ach = 27 * flops / kern_s / 1e12
+    return {"bound": "tensor", "achieved": round(ach, 3), "peak": pk, "unit": "TFLOP/s", "frac": round(ach / pk, 4),
+            "traffic": None, "peak_source": f"{src} 16-bit tensor rate; 27 digit products per FP64 product",
+            "kernel": "k_jk_split", "kernel_ms": round(kern_s * 1e3, 4), "algorithmic_flops": flops}
+
+
 def contraction_roofline(prec, st, m, n, kern_s, alu_peaks, workload="stored_n200_m16"):
     """Roofline of the contraction kernel of one stored build.  FP64 / FP32
     stores: CUDA-core FMAs against the measured FMA rate, counting the
@@ -196,7 +212,7 @@ def sub_stored(fock, W, dev, stream, prec, alu_peaks, steps=20):
         return {"dtype": DTYPES[prec], "ms_per_step": round(ms, 4), "value": round(1e3 / ms, 3),
                 "quartets_per_s": round(st["n_quartets_kept"] / (ms / 1e3), 1), "densities_per_pass": chunk,
                 "setup_ms": round(st["create_ms"], 1), "store_bytes": st["store_bytes"],
-                "roofline": contraction_roofline(prec, st, m, n, ks, alu_peaks)}
+                "roofline": stored_roofline(prec, st, m, n, ks, alu_peaks)}
 
 
 def sub_precision(fock, W, dev, stream, steps=10):
@@ -305,12 +321,18 @@ def sub_df(fock, W, dev, stream, alu_peaks, steps=3):
             ms, ks = timed_builds(fock, fb, m, D, J, K, F, t, stream, steps, 1)
             flops = 2 * 2 * naux * n * n * m + 2 * 2 * naux * n ** 3 * m
             ach = flops / ks / 1e12
+            # FP64 exchange: 28 FP16 digit products per FP64 one (k_df_gemm)
+            _, src, d = peaks()
+            pk = float(d.get("bf16_tflops", 1900.0)) if prec == "fp64" else alu_peaks[prec]
+            ach *= 28 if prec == "fp64" else 1
             rec = {"dtype": DTYPES[prec], "ms_per_step": round(ms, 3), "value": round(1e3 / ms, 3),
                    "setup_ms": round(st["create_ms"], 1), "factor_bytes": st["store_bytes"],
-                   "roofline": {"bound": "alu", "achieved": round(ach, 3), "peak": alu_peaks[prec],
-                                "unit": "TFLOP/s", "frac": round(ach / alu_peaks[prec], 4), "traffic": None,
-                                "peak_source": f"measured {prec.upper()} FMA rate (esmf_measure_fma_peak)",
-                                "kernel": "cuBLAS GEMMs (J: 2, K: 2 per density)",
+                   "roofline": {"bound": "tensor" if prec == "fp64" else "alu", "achieved": round(ach, 3), "peak": pk,
+                                "unit": "TFLOP/s", "frac": round(ach / pk, 4), "traffic": None,
+                                "peak_source": f"{src} 16-bit tensor rate; 28 digit products per FP64 product"
+                                if prec == "fp64" else f"measured {prec.upper()} FMA rate (esmf_measure_fma_peak)",
+                                "kernel": "k_df_gemm (K), cuBLAS GEMMs (J)" if prec == "fp64"
+                                else "cuBLAS GEMMs (J: 2, K: 2 per density)",
                                 "kernel_ms": round(ks * 1e3, 3), "algorithmic_flops": flops}}
             if gd is not None:
                 Jr = np.zeros((m, n, n))
@@ -485,9 +507,9 @@ def run_ours(args):
               "n_occ": es.nocc, "fock_builds_grouped": 3, "precision": args.precision,
               "what": "E, dE/dc0, dE/dsigma, dE/dV (esmf_energy_gradient)",
               # k_gemm_group x5, k_dmax, k_dbank, k_jk_umma, k_finalize_blocked (or
-              # k_jk_cuda, k_finalize), k_energy_fock, k_energy_dots, k_energy_scalars,
+              # k_split_dbank, k_jk_split, k_finalize_blocked; or k_jk_cuda, k_finalize), k_energy_fock, k_energy_dots, k_energy_scalars,
               # k_energy_finish
-              "gpu_launches_per_eval": 13 if split else 11}
+              "gpu_launches_per_eval": 13 if split else 12 if args.precision in ("fp64", "f32x2") else 11}
     # GVP objective (Eq. esmf_gvb) and its derivatives: two grouped passes
     for _ in range(2):
         fb.gvp_gradient(Gd, Vd, Sd, es.c0, es.nocc, -3.0, 0.4, 0.8, stream=stream)
@@ -504,7 +526,7 @@ def run_ours(args):
            "what": "L, E, |grad E|^2, dL/dc0, dL/dsigma, dL/dX (esmf_gvp_gradient)"}
     fb.close()
 
-    roof = contraction_roofline(args.precision, st, m, n, (kern_ms / max(kern_n, 1)) / 1e3, alu_peaks)
+    roof = stored_roofline(args.precision, st, m, n, (kern_ms / max(kern_n, 1)) / 1e3, alu_peaks)
     out = {"metric": METRIC, "value": round(world * 1e3 / ms_step, 3), "unit": UNIT,
            "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
            "ms_per_step": round(ms_step, 4), "higher_is_better": True, "scaling": "weak",
@@ -525,8 +547,9 @@ def run_ours(args):
                    "h2d_bytes_per_step": int(D.numel() * 8),
                    "d2h_bytes_per_step": int(2 * D.numel() * 8 + m * 8)},
            # our kernels per step: tensor path k_dmax, k_dbank, k_jk_umma, k_finalize_blocked;
-           # CUDA-core path k_jk_cuda, k_finalize
-           "gpu_launches": int((4 if split else 2) * args.steps),
+           # FP64 and double-FP32 k_split_dbank, k_jk_split, k_finalize_blocked; CUDA-core
+           # path k_jk_cuda, k_finalize
+           "gpu_launches": int((4 if split else 3 if args.precision in ("fp64", "f32x2") else 2) * args.steps),
            "clocks": clk.summary(),
            "esmf_energy_gradient": energy,
            "esmf_gvp_gradient": gvp}

@@ -210,8 +210,8 @@ int esmf_fock_create_cart(const esmf_basis_t *basis, const int32_t *cart, double
  * tensor cores (14 bytes an element, rows padded to 128 and columns to 64) and
  * 14 bytes an element for the same of as many densities as fit 2.5 GiB (at
  * least one); without room for those, the FP32 layout in FP64 on cuBLAS.
- * FP64: K_k is NaN when D_k holds an infinity, a NaN or an element above 2^500.
- * Errors: INVALID_ARG (bad basis or auxiliary
+ * Densities whose largest element is not in [2^-500, 2^500) take FP64 arithmetic
+ * on CUDA cores there.  Errors: INVALID_ARG (bad basis or auxiliary
  * set, or a metric that is not positive definite), UNSUPPORTED (split 16-bit
  * precisions), OOM, CUDA.
  */

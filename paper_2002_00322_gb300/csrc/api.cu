@@ -1001,12 +1001,21 @@ int esmf_fock_create_df(const esmf_basis_t *basis, const esmf_aux_t *aux, int pr
     if ((rc = df_gemm_fold(h->cublas, naux, (int64_t)nn, Linv, T, B, cs))) return fail(rc);
     if (es == 8) {
         // digit tiles of the factor and of Y for as many densities per pass as fit
-        // 2.5 GiB; without room for them the exchange stays on cuBLAS
+        // 2.5 GiB; without room for them, or with a factor that the digits cannot
+        // hold, the exchange stays on cuBLAS
+        std::vector<int16_t> rows(n);
+        if ((rc = dalloc(h, &h->dfeB, 2 * (size_t)n))) return fail(rc);
+        if ((rc = launch_df_split_rows(B, naux, n, h->dfeB, h->dfeB + n, cs))) return fail(rc);
+        if (cudaMemcpyAsync(rows.data(), h->dfeB, sizeof(int16_t) * n, cudaMemcpyDeviceToHost, cs) ||
+            cudaStreamSynchronize(cs)) {
+            set_error("copy of the factor's row exponents failed");
+            return fail(ESMF_ERR_CUDA);
+        }
         const size_t tb = df_split_tile_bytes(n, naux);
         h->df_group = (int)std::max<size_t>(1, std::min<size_t>(16, ((size_t)5 << 29) / tb));
-        if (cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-            dalloc(h, &h->dfTiles, tb) != ESMF_OK || dalloc(h, &h->dfYt, tb * h->df_group) != ESMF_OK ||
-            dalloc(h, &h->dfeB, 2 * (size_t)n) != ESMF_OK) {
+        if (df_split_rows_fit(n, rows.data()) &&
+            (cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+             dalloc(h, &h->dfTiles, tb) != ESMF_OK || dalloc(h, &h->dfYt, tb * h->df_group) != ESMF_OK)) {
             cudaGetLastError();
             dfree(h, &h->dfTiles, tb);
             dfree(h, &h->dfYt, tb * h->df_group);
@@ -1020,7 +1029,7 @@ int esmf_fock_create_df(const esmf_basis_t *basis, const esmf_aux_t *aux, int pr
         if ((rc = dalloc(h, (unsigned char **)&h->dfB, naux * nn * es))) return fail(rc);
         if ((rc = launch_df_layouts(naux, n, B, 1, h->dfB, h->dfB2, cs))) return fail(rc);
     } else {
-        if (split) rc = launch_df_split_factor(B, naux, n, h->dfeB, h->dfeB + n, h->dfTiles, cs);
+        if (split) rc = launch_df_split_factor(B, naux, n, h->dfeB, h->dfTiles, cs);
         else rc = launch_df_layouts(naux, n, B, 0, nullptr, h->dfB2, cs);
         if (rc) return fail(rc);
         h->dfB = B;                       // the FP64 factor itself is the [P][p][q] layout
@@ -1282,8 +1291,8 @@ int build_df(esmf_fock_t *h, int m, const double *D, double *J, double *K, doubl
     DfSplit sp;
     if (h->dfTiles) {
         sp.n = h->n; sp.naux = h->naux; sp.m = m; sp.group = h->df_group; sp.num_sms = h->num_sms;
-        sp.eB = h->dfeB; sp.nB = h->dfeB + h->n; sp.Btiles = h->dfTiles; sp.D = D;
-        sp.eD = h->dfeD; sp.ED = h->dfED; sp.bad = h->dfED + h->df_m; sp.Dtiles = h->dfDtl; sp.Ytiles = h->dfYt;
+        sp.B = (const double *)h->dfB; sp.eB = h->dfeB; sp.nB = h->dfeB + h->n; sp.Btiles = h->dfTiles; sp.D = D;
+        sp.eD = h->dfeD; sp.ED = h->dfED; sp.top = h->dfED + h->df_m; sp.Dtiles = h->dfDtl; sp.Ytiles = h->dfYt;
         sp.K = (double *)h->dfKt; sp.error = h->err_dev;
     }
     DfBuild a;

@@ -28,6 +28,11 @@
 // t < 6 the error of K against 64-bit references was 5e-13 over 200 functions
 // (DGEMM 3.9e-14).
 //
+// Digits serve densities whose largest element lies in [2^-500, 2^500), where
+// the squares behind the bound on Y stay in FP64's range; k_df_plain takes the
+// others (and those with infinities or NaN) in FP64 arithmetic.  The factor's
+// elements are at most 2^250 (the handle keeps to cuBLAS otherwise).
+//
 // What bounds it: the MMAs (3.6K cycles per block of full size) and the
 // tensor-memory reads after each block (448 of the 512 columns are one
 // accumulator, so they do not overlap).  Sixteen warps read, a quarter of the
@@ -58,6 +63,8 @@ constexpr int DF_SMEM = OFF_CTRL + 1024;
 constexpr int EPI_WARPS = 16;
 constexpr int DF_THREADS = 64 + 32 * EPI_WARPS;
 constexpr int EMIN = 1022 - 600;              // smallest exponent field of a row
+constexpr int DMIN = -500, DMAX = 500;        // exponents of the densities that digits serve
+constexpr int BMAX = 250;                     // largest exponent of the factor
 constexpr uint32_t POLLS = 1u << 22;
 
 struct DfCtrl {
@@ -81,8 +88,13 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float *v) {
     for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// exponent e with |x| < 2^e from the largest exponent field of a row
+// exponent field of x: |x| < 2^(field - 1022)
 __device__ __forceinline__ int exp_field(double x) { return (int)(((uint32_t)__double2hiint(x) >> 20) & 0x7ffu); }
+
+// a density whose largest exponent field is `top` and not served by digits
+__device__ __forceinline__ bool beyond_digits(int top) {
+    return top != 0 && (top > 1022 + DMAX || top <= 1022 + DMIN);
+}
 
 // digits of eight fixed-point values as the eight-element pieces of a tile's
 // group: digit i at dst + i * 2048 (dst addresses the row)
@@ -106,7 +118,9 @@ __device__ __forceinline__ void store_digits(unsigned char *dst, const long long
 
 // ---------------------------------------------------------------- operands
 // eB[p]: exponent of max over P, r of |B[P][p][r]|; nB[p]: exponent above
-// max_P |B_P[p]|_2 (one more, for the rounding of the norm).  One block per p.
+// max_P |B_P[p]|_2 (one more, for the rounding of the norm).  Rows so small that
+// the squares leave FP64's range: |B_P[p]|_2 <= sqrt(n) max |B_P[p][r]|, n < 2^18.
+// One block per p.
 __global__ void __launch_bounds__(256) k_df_brows(const double *B, int naux, int n, int16_t *eB, int16_t *nB) {
     __shared__ double red[8];
     __shared__ int rede[8];
@@ -129,7 +143,7 @@ __global__ void __launch_bounds__(256) k_df_brows(const double *B, int naux, int
     if (threadIdx.x == 0) {
         for (int i = 1; i < 8; ++i) { top = fmax(top, red[i]); e = max(e, rede[i]); }
         eB[p] = (int16_t)(e - 1022);
-        nB[p] = (int16_t)(max(exp_field(sqrt(top)), EMIN) - 1022 + 1);
+        nB[p] = (int16_t)(e < 1022 + DMIN ? e - 1022 + 10 : exp_field(sqrt(top)) - 1022 + 1);
     }
 }
 
@@ -155,22 +169,25 @@ __global__ void k_df_btiles(const double *B, int naux, int n, int npb, int nkb, 
 }
 
 // Per density k and column s: exponent eD[k * ldD + s] of max_r |D_k[r][s]|;
-// per density the exponent above max_s |D_k[:, s]|_2 in ED[k] (EMIN - 1022 at
-// launch) and a flag when an element is not finite or above 2^500.
-__global__ void k_df_dcols(const double *D, int n, int ldD, int16_t *eD, int *ED, int *bad) {
+// per density the exponent above max_s |D_k[:, s]|_2 in ED[k] (any smaller value
+// at launch; the column of the largest element has a norm in range and bounds the
+// columns whose squares underflow) and the exponent field of its largest element
+// in top[k] (0 at launch; subnormal elements count as 1).
+__global__ void k_df_dcols(const double *D, int n, int ldD, int16_t *eD, int *ED, int *top) {
     const int k = blockIdx.y, s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= ldD) return;
-    int e = EMIN;
+    int e = 0;
     double q = 0.0;
     if (s < n)
         for (int r = 0; r < n; ++r) {
             const double v = D[((int64_t)k * n + r) * n + s];
             q = fma(v, v, q);
-            e = max(e, exp_field(v));
+            e = max(e, v != 0.0 ? max(exp_field(v), 1) : 0);
         }
-    eD[(int64_t)k * ldD + s] = (int16_t)(e - 1022);
-    if (e > 1022 + 500) atomicOr(bad + k, 1);
-    else if (s < n) atomicMax(ED + k, max(exp_field(sqrt(q)), EMIN) - 1022 + 1);
+    eD[(int64_t)k * ldD + s] = (int16_t)(max(e, EMIN) - 1022);
+    if (e == 0) return;
+    atomicMax(top + k, e);
+    atomicMax(ED + k, exp_field(sqrt(q)) - 1022 + 1);
 }
 
 // digit tiles of the densities, rows s over r: [k][128 rows s][64 r]
@@ -183,7 +200,7 @@ __global__ void k_df_dtiles(const double *D, int n, int m, int npb, int nkb, int
         const int64_t k = tile / nkb / npb;
         const int s = sb * 128 + row, r0 = kb * 64 + g * 8;
         long long X[8];
-        const int e = s < n ? min(eD[k * ldD + s] + 1022, 1022 + 500) : EMIN;
+        const int e = s < n ? min(eD[k * ldD + s] + 1022, 1022 + DMAX) : EMIN;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const double v = (s < n && r0 + j < n) ? D[(k * n + r0 + j) * n + s] : 0.0;
@@ -199,7 +216,7 @@ struct DfGemm {
     unsigned char *Y;              // first product: tiles of Y out
     double *K;                     // second product: n x n per density, added to
     const int16_t *eB, *nB, *eD;
-    const int *ED, *bad;
+    const int *ED, *top;
     int n, naux, npb, nkb, nsb;    // nsb: blocks of 64 output columns
     int k0, kc, splits, ldD;
     int64_t items;
@@ -364,7 +381,7 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_df_gemm(const __grid_constant
 #pragma unroll
                 for (int i = 0; i < 8; ++i) SH[g][i] = SL[g][i] = 0;
             const int ap = p < G.n ? G.eB[p] : 0;
-            const int yp = p < G.n ? G.nB[p] + G.ED[G.k0 + x.k] : 0;
+            const int yp = p < G.n ? G.nB[p] + G.ED[G.k0 + x.k] : 4096;
             for (int64_t j = x.j0; j < x.j1; ++j, ++blk) {
                 if (!__all_sync(~0u, wait_for(&c.accfull, blk & 1, abort_flag))) { fail(44); ok = false; break; }
                 tc_fence_after();
@@ -394,17 +411,16 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_df_gemm(const __grid_constant
             }
             if (SECOND && ok) {
                 const int k = G.k0 + x.k;
-                const bool bad = G.bad[k] != 0;
+                const bool plain = beyond_digits(G.top[k]);
 #pragma unroll
                 for (int g = 0; g < 2; ++g)
-                    if (g < groups)
+                    if (g < groups && !plain)
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const int q = x.ob * 64 + (ch + 4 * g) * 8 + i;
                             if (p < G.n && q < G.n) {
                                 const double y = fma((double)SH[g][i], 0x1p36, (double)SL[g][i]);
-                                atomicAdd(G.K + ((int64_t)k * G.n + p) * G.n + q,
-                                          bad ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(y, yp + G.eB[q] - 70));
+                                atomicAdd(G.K + ((int64_t)k * G.n + p) * G.n + q, scalbn(y, yp + G.eB[q] - 70));
                             }
                         }
             }
@@ -419,9 +435,11 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_df_gemm(const __grid_constant
                         long long X[8];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
-                            const int r = yp - ap - ed[g * 32 + i] + 70 - BITS;    // right shift, >= 6
+                            // right shift: nB > eB and ED > eD make it 10 at least (rows beyond n and
+                            // densities that k_df_plain takes get zeros)
+                            const int r = yp - ap - ed[g * 32 + i] + 70 - BITS;
                             const __int128 S = ((__int128)SH[g][i] << 36) + SL[g][i];
-                            X[i] = r > 100 ? 0 : (long long)((S + ((__int128)1 << (max(r, 1) - 1))) >> max(r, 1));
+                            X[i] = r > 100 || r < 1 ? 0 : (long long)((S + ((__int128)1 << (r - 1))) >> r);
                         }
                         store_digits(out + 4 * g * GROUP, X);
                     }
@@ -434,6 +452,44 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_df_gemm(const __grid_constant
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, 512);
+    }
+}
+
+// K of the densities beyond the digits' range, in FP64 arithmetic: a block forms
+// whole rows p, y[s] = sum_r B[P][p][r] D[r][s] for a piece of s at a time, then
+// K[p][q] += sum_s y[s] B[P][s][q] (B is symmetric; both sums read whole rows).
+// Others return at once.  200 functions, 700 auxiliaries: 34 ms a density (the
+// two cuBLAS products took 27 ms), FP64-bound.
+__global__ void __launch_bounds__(256) k_df_plain(const double *B, const double *D, int n, int naux, int m,
+                                                  const int *top, double *K) {
+    constexpr int PIECE = 1024;
+    __shared__ double y[PIECE];
+    const int64_t nn = (int64_t)n * n;
+    for (int k = 0; k < m; ++k) {
+        if (!beyond_digits(top[k])) continue;
+        const double *Dk = D + k * nn;
+        for (int p = blockIdx.x; p < n; p += gridDim.x) {
+            double *Kp = K + k * nn + (int64_t)p * n;
+            for (int q = threadIdx.x; q < n; q += blockDim.x) Kp[q] = 0.0;
+            for (int P = 0; P < naux; ++P) {
+                const double *BP = B + P * nn, *bp = BP + (int64_t)p * n;
+                for (int s0 = 0; s0 < n; s0 += PIECE) {
+                    const int len = min(PIECE, n - s0);
+                    __syncthreads();
+                    for (int s = threadIdx.x; s < len; s += blockDim.x) {
+                        double a = 0.0;
+                        for (int r = 0; r < n; ++r) a = fma(bp[r], Dk[(int64_t)r * n + s0 + s], a);
+                        y[s] = a;
+                    }
+                    __syncthreads();
+                    for (int q = threadIdx.x; q < n; q += blockDim.x) {
+                        double a = Kp[q];
+                        for (int s = 0; s < len; ++s) a = fma(y[s], BP[(int64_t)(s0 + s) * n + q], a);
+                        Kp[q] = a;
+                    }
+                }
+            }
+        }
     }
 }
 
@@ -468,9 +524,19 @@ int df_gemm(const DfGemm &g, int num_sms, cudaStream_t s) {
 
 size_t df_split_tile_bytes(int n, int64_t matrices) { return (size_t)matrices * row_blocks(n) * sum_blocks(n) * TILE; }
 
-int launch_df_split_factor(const double *B, int naux, int n, int16_t *eB, int16_t *nB, unsigned char *tiles, cudaStream_t s) {
+int launch_df_split_rows(const double *B, int naux, int n, int16_t *eB, int16_t *nB, cudaStream_t s) {
     k_df_brows<<<n, 256, 0, s>>>(B, naux, n, eB, nB);
     CKS(cudaGetLastError());
+    return ESMF_OK;
+}
+
+bool df_split_rows_fit(int n, const int16_t *eB) {
+    int top = EMIN - 1022;
+    for (int p = 0; p < n; ++p) top = eB[p] > top ? eB[p] : top;
+    return top >= -BMAX && top <= BMAX;
+}
+
+int launch_df_split_factor(const double *B, int naux, int n, const int16_t *eB, unsigned char *tiles, cudaStream_t s) {
     const int npb = row_blocks(n), nkb = sum_blocks(n);
     k_df_btiles<<<grid_for((int64_t)naux * npb * nkb * 1024), 256, 0, s>>>(B, naux, n, npb, nkb, eB, tiles);
     CKS(cudaGetLastError());
@@ -481,16 +547,15 @@ int launch_df_split_exchange(const DfSplit &a, cudaStream_t s) {
     const int n = a.n, npb = row_blocks(n), nkb = sum_blocks(n), ldD = nkb * 64;
     const int64_t nn = (int64_t)n * n;
     CKS(cudaMemsetAsync(a.K, 0, sizeof(double) * a.m * nn, s));
-    CKS(cudaMemsetAsync(a.bad, 0, sizeof(int) * a.m, s));
-    // EMIN - 1022 = -600 is not a repeated byte; any smaller start does for the maximum
+    CKS(cudaMemsetAsync(a.top, 0, sizeof(int) * a.m, s));
     CKS(cudaMemsetAsync(a.ED, 0x80, sizeof(int) * a.m, s));
-    k_df_dcols<<<dim3((ldD + 63) / 64, a.m), 64, 0, s>>>(a.D, n, ldD, a.eD, a.ED, a.bad);
+    k_df_dcols<<<dim3((ldD + 63) / 64, a.m), 64, 0, s>>>(a.D, n, ldD, a.eD, a.ED, a.top);
     CKS(cudaGetLastError());
     k_df_dtiles<<<grid_for((int64_t)a.m * npb * nkb * 1024), 256, 0, s>>>(a.D, n, a.m, npb, nkb, ldD, a.eD, a.Dtiles);
     CKS(cudaGetLastError());
     for (int k0 = 0; k0 < a.m; k0 += a.group) {
         DfGemm g;
-        g.eB = a.eB; g.nB = a.nB; g.eD = a.eD; g.ED = a.ED; g.bad = a.bad;
+        g.eB = a.eB; g.nB = a.nB; g.eD = a.eD; g.ED = a.ED; g.top = a.top;
         g.n = n; g.naux = a.naux; g.npb = npb; g.nkb = nkb; g.nsb = nkb; g.ldD = ldD;
         g.k0 = k0; g.kc = a.m - k0 < a.group ? a.m - k0 : a.group;
         g.Y = a.Ytiles; g.K = a.K; g.error = a.error;
@@ -508,6 +573,8 @@ int launch_df_split_exchange(const DfSplit &a, cudaStream_t s) {
         rc = df_gemm<true>(g, a.num_sms, s);
         if (rc != ESMF_OK) return rc;
     }
+    k_df_plain<<<n < 4 * a.num_sms ? n : 4 * a.num_sms, 256, 0, s>>>(a.B, a.D, n, a.naux, a.m, a.top, a.K);
+    CKS(cudaGetLastError());
     return ESMF_OK;
 }
 

@@ -180,18 +180,22 @@ size_t split_jbank_bytes(int nb);
 // ---- df_split.cu (density-fitted exchange on the tensor cores, FP64 accuracy)
 struct DfSplit {
     int n, naux, m, group, num_sms;              // group: densities per pass over the Y tiles
-    const int16_t *eB, *nB;                      // row exponents of the factor
+    const double *B;                             // the fitted factor [P][p][q]
+    const int16_t *eB, *nB;                      // its row exponents
     const unsigned char *Btiles;
     const double *D;
     int16_t *eD;                                 // work: column exponents, m x 64 ceil(n / 64)
-    int *ED, *bad;                               // work: per density
+    int *ED, *top;                               // work: per density
     unsigned char *Dtiles, *Ytiles;              // work: m matrices, group * naux matrices
     double *K;                                   // m x n x n
     int *error;                                  // device error flag, 0 = ok
 };
 size_t df_split_tile_bytes(int n, int64_t matrices);
-// row exponents (n each) and digit tiles (naux matrices) of the fitted factor B[P][p][q]
-int launch_df_split_factor(const double *B, int naux, int n, int16_t *eB, int16_t *nB, unsigned char *tiles, cudaStream_t s);
+// row exponents (n each) of the fitted factor B[P][p][q], whether digits can hold
+// the factor (host copy of eB), and its digit tiles (naux matrices)
+int launch_df_split_rows(const double *B, int naux, int n, int16_t *eB, int16_t *nB, cudaStream_t s);
+bool df_split_rows_fit(int n, const int16_t *eB);
+int launch_df_split_factor(const double *B, int naux, int n, const int16_t *eB, unsigned char *tiles, cudaStream_t s);
 int launch_df_split_exchange(const DfSplit &a, cudaStream_t s);
 
 // ---- df.cu (density-fitted J and K)

@@ -18,12 +18,15 @@
 // bounds the rows, so no pass over Y is needed to find their exponents.
 //
 // k_df_gemm forms tiles of 128 x 64 outputs.  For each block of 64 summed
-// elements the digit products with i + j = t < 7 are summed exactly in FP32
-// tensor memory (7 x 64 columns), read and added to two 64-bit integers per
-// output in registers, SH for t < 3 and SL for the rest: a product is
-// 2^(e_a + e_b - 70) (2^36 SH + SL), and nothing is rounded until all blocks are
-// summed (an integer holds 2^11 blocks at least; each CTA's range is shorter).
-// The digit pairs left out weigh 2^-63 of the rows' largest product.  A row
+// elements the digit products with i + j = t < 7 are summed in FP32 tensor
+// memory (7 x 64 columns), read and added to two 64-bit integers per output in
+// registers, SH for t < 3 and SL for the rest: a product is
+// 2^(e_a + e_b - 70) (2^36 SH + SL).  The sums of a block are exact for t <= 3 (at
+// most 4 * 64 terms of 2^16, below 2^24 or equal); those of t >= 4 are too unless
+// their digits line up (up to 7 * 64 terms of 2^16), and an addition above 2^24
+// then rounds by 1, 2^-52 of the rows' largest product.  A block adds at most
+// 2^51 + 2^43 to SL, so the integers hold 2048 blocks, and no CTA sums more
+// (df_ranges).  The digit pairs left out weigh 2^-63 of that product each.  A row
 // spans all auxiliaries, whose elements differ by decades: with six digits and
 // t < 6 the error of K against 64-bit references was 5e-13 over 200 functions
 // (DGEMM 3.9e-14).
@@ -65,6 +68,7 @@ constexpr int DF_THREADS = 64 + 32 * EPI_WARPS;
 constexpr int EMIN = 1022 - 600;              // smallest exponent field of a row
 constexpr int DMIN = -500, DMAX = 500;        // exponents of the densities that digits serve
 constexpr int BMAX = 250;                     // largest exponent of the factor
+constexpr int MAX_BLOCKS = 2048;              // blocks of 64 summed elements that SL and SH hold
 constexpr uint32_t POLLS = 1u << 22;
 
 struct DfCtrl {
@@ -512,6 +516,16 @@ int grid_for(int64_t work) {
     return (int)(g < 1 ? 1 : (g > 152 * 32 ? 152 * 32 : g));
 }
 
+// Ranges that the naux * sum_blocks(n) summed blocks of the second product are
+// cut into: about four items per SM, 4 blocks or more each, never above MAX_BLOCKS.
+int df_ranges(int n, int naux, int kc, int num_sms) {
+    const int64_t tiles = (int64_t)kc * row_blocks(n) * sum_blocks(n), blocks = (int64_t)naux * sum_blocks(n);
+    int64_t sp = (4 * num_sms + tiles - 1) / tiles;
+    if (sp > blocks / 4) sp = blocks / 4;
+    const int64_t least = (blocks + MAX_BLOCKS - 1) / MAX_BLOCKS;
+    return (int)(sp < least ? least : sp);
+}
+
 template <bool SECOND>
 int df_gemm(const DfGemm &g, int num_sms, cudaStream_t s) {
     CKS(cudaFuncSetAttribute(k_df_gemm<SECOND>, cudaFuncAttributeMaxDynamicSharedMemorySize, DF_SMEM));
@@ -521,6 +535,9 @@ int df_gemm(const DfGemm &g, int num_sms, cudaStream_t s) {
 }
 
 }  // namespace
+
+// df_ranges for the tests
+extern "C" int esmf_df_exchange_ranges(int n, int naux, int kc, int num_sms) { return df_ranges(n, naux, kc, num_sms); }
 
 size_t df_split_tile_bytes(int n, int64_t matrices) { return (size_t)matrices * row_blocks(n) * sum_blocks(n) * TILE; }
 
@@ -533,7 +550,7 @@ int launch_df_split_rows(const double *B, int naux, int n, int16_t *eB, int16_t 
 bool df_split_rows_fit(int n, const int16_t *eB) {
     int top = EMIN - 1022;
     for (int p = 0; p < n; ++p) top = eB[p] > top ? eB[p] : top;
-    return top >= -BMAX && top <= BMAX;
+    return top >= -BMAX && top <= BMAX && sum_blocks(n) <= MAX_BLOCKS;
 }
 
 int launch_df_split_factor(const double *B, int naux, int n, const int16_t *eB, unsigned char *tiles, cudaStream_t s) {
@@ -563,13 +580,9 @@ int launch_df_split_exchange(const DfSplit &a, cudaStream_t s) {
         g.items = (int64_t)a.naux * npb * g.kc * nkb;
         int rc = df_gemm<false>(g, a.num_sms, s);
         if (rc != ESMF_OK) return rc;
-        // ranges of the summed blocks for about four items per SM, 4 blocks or more each
-        const int64_t tiles = (int64_t)g.kc * npb * nkb, blocks = (int64_t)a.naux * nkb;
-        int64_t sp = (4 * a.num_sms + tiles - 1) / tiles;
-        if (sp > blocks / 4) sp = blocks / 4;
-        g.splits = (int)(sp < 1 ? 1 : sp);
+        g.splits = df_ranges(n, a.naux, g.kc, a.num_sms);
         g.A = a.Ytiles; g.B = a.Btiles;
-        g.items = tiles * g.splits;
+        g.items = (int64_t)g.kc * npb * nkb * g.splits;
         rc = df_gemm<true>(g, a.num_sms, s);
         if (rc != ESMF_OK) return rc;
     }

@@ -84,7 +84,7 @@ struct esmf_fock {
     int df_m = 0;
     // FP64 exchange by digit splitting (df_split.cu), used when dfTiles is set:
     // the factor's digit tiles and row exponents, per-build work
-    unsigned char *dfTiles = nullptr, *dfYt = nullptr, *dfDtl = nullptr;
+    unsigned char *dfTiles = nullptr, *dfYt = nullptr, *dfDtl = nullptr, *dfS = nullptr;
     int16_t *dfeB = nullptr, *dfeD = nullptr;
     int *dfED = nullptr;
     int df_group = 0;
@@ -282,7 +282,7 @@ void release(esmf_fock *h) {
     cudaFree(h->dw); cudaFree(h->dwb);
     cudaFree(h->dfB); cudaFree(h->dfB2); cudaFree(h->dfDt); cudaFree(h->dfJt); cudaFree(h->dfKt);
     cudaFree(h->dfg); cudaFree(h->dfY);
-    cudaFree(h->dfTiles); cudaFree(h->dfYt); cudaFree(h->dfDtl); cudaFree(h->dfeB); cudaFree(h->dfeD); cudaFree(h->dfED);
+    cudaFree(h->dfTiles); cudaFree(h->dfYt); cudaFree(h->dfS); cudaFree(h->dfDtl); cudaFree(h->dfeB); cudaFree(h->dfeD); cudaFree(h->dfED);
     cudaFree(h->thcX); cudaFree(h->thcZ); cudaFree(h->thcDt); cudaFree(h->thcA); cudaFree(h->thcM);
     cudaFree(h->thcy); cudaFree(h->thcz); cudaFree(h->thcJt); cudaFree(h->thcKt);
     df_cublas_destroy(h->cublas);
@@ -1015,7 +1015,8 @@ int esmf_fock_create_df(const esmf_basis_t *basis, const esmf_aux_t *aux, int pr
         h->df_group = (int)std::max<size_t>(1, std::min<size_t>(16, ((size_t)5 << 29) / tb));
         if (df_split_rows_fit(n, rows.data()) &&
             (cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-             dalloc(h, &h->dfTiles, tb) != ESMF_OK || dalloc(h, &h->dfYt, tb * h->df_group) != ESMF_OK)) {
+             dalloc(h, &h->dfTiles, tb) != ESMF_OK || dalloc(h, &h->dfYt, tb * h->df_group) != ESMF_OK ||
+             dalloc(h, &h->dfS, df_split_sum_bytes(n, h->df_group)) != ESMF_OK)) {
             cudaGetLastError();
             dfree(h, &h->dfTiles, tb);
             dfree(h, &h->dfYt, tb * h->df_group);
@@ -1292,7 +1293,7 @@ int build_df(esmf_fock_t *h, int m, const double *D, double *J, double *K, doubl
     if (h->dfTiles) {
         sp.n = h->n; sp.naux = h->naux; sp.m = m; sp.group = h->df_group; sp.num_sms = h->num_sms;
         sp.B = (const double *)h->dfB; sp.eB = h->dfeB; sp.nB = h->dfeB + h->n; sp.Btiles = h->dfTiles; sp.D = D;
-        sp.eD = h->dfeD; sp.ED = h->dfED; sp.top = h->dfED + h->df_m; sp.Dtiles = h->dfDtl; sp.Ytiles = h->dfYt;
+        sp.eD = h->dfeD; sp.ED = h->dfED; sp.top = h->dfED + h->df_m; sp.Dtiles = h->dfDtl; sp.Ytiles = h->dfYt; sp.S = (unsigned long long *)h->dfS;
         sp.K = (double *)h->dfKt; sp.error = h->err_dev;
     }
     DfBuild a;

@@ -68,6 +68,7 @@ constexpr int DF_THREADS = 64 + 32 * EPI_WARPS;
 constexpr int EMIN = 1022 - 600;              // smallest exponent field of a row
 constexpr int DMIN = -500, DMAX = 500;        // exponents of the densities that digits serve
 constexpr int BMAX = 250;                     // largest exponent of the factor
+constexpr unsigned long long SL_MASK = (1ull << 36) - 1;   // SL below 2^36 SH
 constexpr int MAX_BLOCKS = 2048;              // blocks of 64 summed elements that SL and SH hold
 constexpr uint32_t POLLS = 1u << 22;
 
@@ -218,7 +219,7 @@ __global__ void k_df_dtiles(const double *D, int n, int m, int npb, int nkb, int
 struct DfGemm {
     const unsigned char *A, *B;    // digit tiles of the two operands
     unsigned char *Y;              // first product: tiles of Y out
-    double *K;                     // second product: n x n per density, added to
+    unsigned long long *S;         // second product: SH, then SL, n x n per density of the group, added to
     const int16_t *eB, *nB, *eD;
     const int *ED, *top;
     int n, naux, npb, nkb, nsb;    // nsb: blocks of 64 output columns
@@ -414,17 +415,17 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_df_gemm(const __grid_constant
                 if (lane == 0) mbar_arrive(&c.accfree);
             }
             if (SECOND && ok) {
-                const int k = G.k0 + x.k;
-                const bool plain = beyond_digits(G.top[k]);
 #pragma unroll
                 for (int g = 0; g < 2; ++g)
-                    if (g < groups && !plain)
+                    if (g < groups)
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const int q = x.ob * 64 + (ch + 4 * g) * 8 + i;
                             if (p < G.n && q < G.n) {
-                                const double y = fma((double)SH[g][i], 0x1p36, (double)SL[g][i]);
-                                atomicAdd(G.K + ((int64_t)k * G.n + p) * G.n + q, scalbn(y, yp + G.eB[q] - 70));
+                                // the ranges' sums join as integers: any order gives the same bits
+                                unsigned long long *o = G.S + ((int64_t)x.k * G.n + p) * G.n + q;
+                                atomicAdd(o, (unsigned long long)(SH[g][i] + (SL[g][i] >> 36)));
+                                atomicAdd(o + (int64_t)G.kc * G.n * G.n, (unsigned long long)SL[g][i] & SL_MASK);
                             }
                         }
             }
@@ -456,6 +457,20 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_df_gemm(const __grid_constant
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, 512);
+    }
+}
+
+// K of a group's densities from their integer sums (each range adds less than
+// 2^36 to SL, and 2^18 blocks, more than the device has room for, 2^59 to SH)
+__global__ void k_df_kout(const __grid_constant__ DfGemm G, double *K) {
+    const int p = blockIdx.x, k = G.k0 + blockIdx.y;
+    if (beyond_digits(G.top[k])) return;
+    const unsigned long long *row = G.S + ((int64_t)blockIdx.y * G.n + p) * G.n;
+    const int e = G.nB[p] + G.ED[k] - 70;
+    for (int q = threadIdx.x; q < G.n; q += blockDim.x) {
+        const unsigned long long lo = row[q + (int64_t)G.kc * G.n * G.n];
+        const long long hi = (long long)(row[q] + (lo >> 36));
+        K[((int64_t)k * G.n + p) * G.n + q] = scalbn(fma((double)hi, 0x1p36, (double)(lo & SL_MASK)), e + G.eB[q]);
     }
 }
 
@@ -541,6 +556,8 @@ extern "C" int esmf_df_exchange_ranges(int n, int naux, int kc, int num_sms) { r
 
 size_t df_split_tile_bytes(int n, int64_t matrices) { return (size_t)matrices * row_blocks(n) * sum_blocks(n) * TILE; }
 
+size_t df_split_sum_bytes(int n, int group) { return (size_t)group * n * n * 2 * sizeof(unsigned long long); }
+
 int launch_df_split_rows(const double *B, int naux, int n, int16_t *eB, int16_t *nB, cudaStream_t s) {
     k_df_brows<<<n, 256, 0, s>>>(B, naux, n, eB, nB);
     CKS(cudaGetLastError());
@@ -562,8 +579,6 @@ int launch_df_split_factor(const double *B, int naux, int n, const int16_t *eB, 
 
 int launch_df_split_exchange(const DfSplit &a, cudaStream_t s) {
     const int n = a.n, npb = row_blocks(n), nkb = sum_blocks(n), ldD = nkb * 64;
-    const int64_t nn = (int64_t)n * n;
-    CKS(cudaMemsetAsync(a.K, 0, sizeof(double) * a.m * nn, s));
     CKS(cudaMemsetAsync(a.top, 0, sizeof(int) * a.m, s));
     CKS(cudaMemsetAsync(a.ED, 0x80, sizeof(int) * a.m, s));
     k_df_dcols<<<dim3((ldD + 63) / 64, a.m), 64, 0, s>>>(a.D, n, ldD, a.eD, a.ED, a.top);
@@ -575,7 +590,7 @@ int launch_df_split_exchange(const DfSplit &a, cudaStream_t s) {
         g.eB = a.eB; g.nB = a.nB; g.eD = a.eD; g.ED = a.ED; g.top = a.top;
         g.n = n; g.naux = a.naux; g.npb = npb; g.nkb = nkb; g.nsb = nkb; g.ldD = ldD;
         g.k0 = k0; g.kc = a.m - k0 < a.group ? a.m - k0 : a.group;
-        g.Y = a.Ytiles; g.K = a.K; g.error = a.error;
+        g.Y = a.Ytiles; g.S = a.S; g.error = a.error;
         g.A = a.Btiles; g.B = a.Dtiles; g.splits = 1;
         g.items = (int64_t)a.naux * npb * g.kc * nkb;
         int rc = df_gemm<false>(g, a.num_sms, s);
@@ -583,8 +598,11 @@ int launch_df_split_exchange(const DfSplit &a, cudaStream_t s) {
         g.splits = df_ranges(n, a.naux, g.kc, a.num_sms);
         g.A = a.Ytiles; g.B = a.Btiles;
         g.items = (int64_t)g.kc * npb * nkb * g.splits;
+        CKS(cudaMemsetAsync(a.S, 0, df_split_sum_bytes(n, g.kc), s));
         rc = df_gemm<true>(g, a.num_sms, s);
         if (rc != ESMF_OK) return rc;
+        k_df_kout<<<dim3(n, g.kc), n <= 128 ? 128 : 256, 0, s>>>(g, a.K);
+        CKS(cudaGetLastError());
     }
     k_df_plain<<<n < 4 * a.num_sms ? n : 4 * a.num_sms, 256, 0, s>>>(a.B, a.D, n, a.naux, a.m, a.top, a.K);
     CKS(cudaGetLastError());

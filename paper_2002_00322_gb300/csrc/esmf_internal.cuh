@@ -187,10 +187,12 @@ struct DfSplit {
     int16_t *eD;                                 // work: column exponents, m x 64 ceil(n / 64)
     int *ED, *top;                               // work: per density
     unsigned char *Dtiles, *Ytiles;              // work: m matrices, group * naux matrices
+    unsigned long long *S;                       // work: df_split_sum_bytes(n, group)
     double *K;                                   // m x n x n
     int *error;                                  // device error flag, 0 = ok
 };
 size_t df_split_tile_bytes(int n, int64_t matrices);
+size_t df_split_sum_bytes(int n, int group);
 // row exponents (n each) of the fitted factor B[P][p][q], whether digits can hold
 // the factor (host copy of eB), and its digit tiles (naux matrices)
 int launch_df_split_rows(const double *B, int naux, int n, int16_t *eB, int16_t *nB, cudaStream_t s);

@@ -116,7 +116,7 @@ struct esmf_fock {
     int *err_host = nullptr, *err_dev = nullptr;   // mapped page-locked flag
     int64_t n_stored = 0, store_bytes = 0, n_kept_unique = 0;
     // work (device): the FP64 accumulators of a build of m <= work_m densities,
-    // J then K (then, on the split path, K's transposed blocks and a flag word)
+    // J then K (then, on the split path, K's transposed blocks and an int a density)
     double *acc = nullptr;
     size_t acc_n = 0;
     // FP64 and double-FP32: density digit tiles of the tensor-core path;
@@ -329,7 +329,7 @@ bool split_path(const esmf_fock *h) {
 // doubles of the accumulators of a build of m densities
 size_t acc_doubles(const esmf_fock *h, int m) {
     const size_t cnt = (size_t)m * h->np * h->np;
-    return split_path(h) ? 3 * cnt + 1 : 2 * cnt;
+    return split_path(h) ? 3 * cnt + (m + 1) / 2 : 2 * cnt;
 }
 
 int ensure_work(esmf_fock *h, int m) {
@@ -1438,7 +1438,7 @@ int build_range(esmf_fock_t *h, int64_t b0, int64_t b1, int m, const double *D, 
             L.kbank = h->skbank; L.jbank = h->sjbank; L.D = D; L.n = h->n; L.nb = h->nb; L.m = m;
             L.num_sms = h->num_sms;
             L.Jacc = Jacc; L.Kacc = Kacc; L.KTacc = Kacc + cnt;
-            L.nonfinite = (int *)(Kacc + 2 * cnt); L.error = h->err_dev;
+            L.top = (int *)(Kacc + 2 * cnt); L.error = h->err_dev;
             if (h->mode == ESMF_MODE_STORED) {
                 L.ev_start = e0; L.ev_stop = e1;
                 RET(launch_jk_split(L, s));

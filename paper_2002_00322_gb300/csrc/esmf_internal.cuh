@@ -169,7 +169,7 @@ struct SplitLaunch {
     const double *D;
     int n, nb, m, num_sms;
     double *Jacc, *Kacc, *KTacc; // block-major accumulators [X][Y][k][x][y]
-    int *nonfinite;              // device flag, zero at launch
+    int *top;                    // m ints, zero at launch: largest exponent fields of the densities
     int *error;                  // device error flag, 0 = ok
     cudaEvent_t ev_start = nullptr, ev_stop = nullptr;
 };

@@ -27,7 +27,7 @@ template <int BITS>
 __device__ __forceinline__ long long fixed_point_f(float x, int emax) {
     const uint32_t b = __float_as_uint(x);
     const int e = (int)((b >> 23) & 0xffu);
-    const int sh = min(emax - 896 - e, 63);
+    const int sh = min(emax - 896 - max(e, 1), 63);      // subnormal parts have the exponent of field 1
     const unsigned long long mant = (b & 0x7fffffu) | (e ? 0x800000u : 0u);
     const unsigned long long r = (((mant << (BITS - 23)) >> sh) + 1) >> 1;
     const long long sg = (int)b >> 31;

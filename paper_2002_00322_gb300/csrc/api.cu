@@ -332,16 +332,27 @@ size_t acc_doubles(const esmf_fock *h, int m) {
     return split_path(h) ? 3 * cnt + (m + 1) / 2 : 2 * cnt;
 }
 
-int ensure_work(esmf_fock *h, int m) {
-    if (split_path(h) && !h->skbank) {
-        // without room for the digit tiles the handle keeps the CUDA-core kernel
-        if (dalloc(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb)) != ESMF_OK ||
-            dalloc(h, (unsigned char **)&h->sjbank, split_jbank_bytes(h->nb)) != ESMF_OK) {
-            cudaGetLastError();
-            dfree(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb));
-            h->no_split = true;
-        }
+// Gives the digit-splitting path up where its memory does not fit: all that it
+// holds goes back, and the handle's builds take the CUDA-core kernel, which needs
+// none of it.
+void drop_split(esmf_fock *h) {
+    cudaGetLastError();
+    dfree(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb));
+    dfree(h, (unsigned char **)&h->sjbank, split_jbank_bytes(h->nb));
+    if (h->mode == ESMF_MODE_DIRECT) {
+        dfree(h, (unsigned char **)&h->scratch, (size_t)h->scratch_bytes);
+        dfree(h, &h->offsets, h->nbricks + 1);
+        h->scratch_bytes = 0;
+        h->chunks.clear();
     }
+    h->no_split = true;
+}
+
+int ensure_work(esmf_fock *h, int m) {
+    if (split_path(h) && !h->skbank &&
+        (dalloc(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb)) != ESMF_OK ||
+         dalloc(h, (unsigned char **)&h->sjbank, split_jbank_bytes(h->nb)) != ESMF_OK))
+        drop_split(h);
     if ((h->mode == ESMF_MODE_STORED || tensor_direct(h)) && is_split16(h->prec) && !h->kbank) {
         RET(dalloc(h, (unsigned char **)&h->kbank, umma_kbank_bytes(h->nb)));
         RET(dalloc(h, (unsigned char **)&h->jbank, umma_jbank_bytes(h->nb)));
@@ -358,10 +369,7 @@ int ensure_work(esmf_fock *h, int m) {
     dfree(h, (unsigned char **)&h->Dt, (size_t)h->work_m * h->n * h->n * tb);
     h->work_m = 0;
     h->acc_n = 0;
-    if (split_path(h) && dalloc(h, &h->acc, acc_doubles(h, m)) != ESMF_OK) {
-        cudaGetLastError();
-        h->no_split = true;
-    }
+    if (split_path(h) && dalloc(h, &h->acc, acc_doubles(h, m)) != ESMF_OK) drop_split(h);
     if (!h->acc) RET(dalloc(h, &h->acc, acc_doubles(h, m)));
     h->acc_n = acc_doubles(h, m);
     if (tb) RET(dalloc(h, (unsigned char **)&h->Dt, (size_t)m * h->n * h->n * tb));

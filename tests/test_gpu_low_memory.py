@@ -1,0 +1,53 @@
+"""FP64 handles on a device with little memory left: the memory of the digit-
+splitting paths is optional, so a build or create that fits without it succeeds.
+
+The device's free memory is taken by one plain allocation; the sizes below
+leave some hundred MB.
+"""
+import numpy as np
+import pytest
+
+from paper_2002_00322_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+MB = 1 << 20
+
+
+def hog(leave):
+    """All but `leave` bytes of the device's free memory."""
+    import torch
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
+
+
+def close(got, ref, tol):
+    for x, r in zip(got, ref):
+        assert np.linalg.norm(x - r) <= tol * np.linalg.norm(r)
+
+
+def test_third_accumulator_does_not_fit(esmf):
+    """Digit tiles and two accumulators do not fit together, two accumulators do."""
+    import torch
+    n, m = 800, 64
+    w = W.small_random(n, 1, 3, tol=1e-6, edge=400.0)             # a thin gas: few bricks
+    D = torch.randn((m, n, n), dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    J, K = torch.empty_like(D), torch.empty_like(D)
+    tiles = 100 * 100 * (6 * 2 * 16 * 128 + 32) + 50 * 101 * (6 * 16 * 128 + 32)
+    acc = m * n * n * 8
+    with esmf.FockBuilder(w.basis, w.tol, "stored", "fp64") as fb:
+        fb.set_path("cuda_core")
+        ref = [x.cpu().numpy() for x in fb.build(D[:2])[:2]]      # loads the kernels
+        fb.set_path("auto")
+        fb.build(D[:2])
+    with esmf.FockBuilder(w.basis, w.tol, "stored", "fp64") as fb:
+        fill = hog(2 * acc + tiles // 2)
+        try:
+            fb.build(D, J, K, want_traces=False)
+            used = fb.stats()["device_bytes"]
+            fb.build(D, J, K, want_traces=False)
+            assert fb.stats()["device_bytes"] == used
+        finally:
+            del fill
+            torch.cuda.empty_cache()
+        close([x[:2].cpu().numpy() for x in (J, K)], ref, 1e-11)

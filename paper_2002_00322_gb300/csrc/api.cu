@@ -771,64 +771,6 @@ static int create_impl(const esmf_basis_t *basis, const int32_t *cart, double to
                 return fail(ESMF_ERR_CUDA);
             h->nparts = (int)parts.size() - 1;
         }
-        if (use_mode == ESMF_MODE_DIRECT && h->prec != ESMF_PREC_FP32 && !h->cart) {
-            // integral-direct on the tensor cores: chunks of whole items whose
-            // records fit the scratch buffer (2 GiB, or a quarter of the budget;
-            // an item larger than that is a chunk of its own).  FP64 handles
-            // take it when their budget and memory hold it and the density digits
-            // too, and evaluate in the contraction kernel otherwise.
-            const bool by_split = !is_split16(h->prec);
-            const int eb = elem_bytes(h->prec);
-            int64_t cap = (int64_t)2 << 30;
-            if (budget_bytes > 0) cap = std::min<int64_t>(cap, budget_bytes / 4);
-            const int64_t nk = h->nbricks;
-            std::vector<int64_t> ch{0};
-            int64_t prev = 0;                        // the last item start seen
-            for (int64_t i = 1; i <= nk; ++i) {
-                if (i < nk && !(kept[i].pad & BRICK_ITEM_FIRST)) continue;
-                if ((offs[i] - offs[ch.back()]) * eb > cap && prev > ch.back()) ch.push_back(prev);
-                prev = i;
-            }
-            if (ch.back() != nk) ch.push_back(nk);
-            std::vector<int64_t> roff(nk + 1, 0);
-            int64_t most = 0;
-            for (size_t c = 0; c + 1 < ch.size(); ++c) {
-                for (int64_t i = ch[c]; i < ch[c + 1]; ++i) roff[i] = offs[i] - offs[ch[c]];
-                most = std::max(most, (offs[ch[c + 1]] - offs[ch[c]]) * eb);
-            }
-            h->chunks = ch;
-            bool room = true;
-            if (by_split) {
-                const int64_t need = most + (nk + 1) * 8 + (int64_t)split_kbank_bytes(h->nb) +
-                                     (int64_t)split_jbank_bytes(h->nb);
-                room = !h->no_split && (budget_bytes == 0 || h->device_bytes + need <= budget_bytes);
-                if (room && dalloc(h, (unsigned char **)&h->scratch, (size_t)most) != ESMF_OK) {
-                    cudaGetLastError();
-                    room = false;
-                }
-            } else if ((rc = dalloc(h, (unsigned char **)&h->scratch, (size_t)most))) {
-                return fail(rc);
-            }
-            if (room) {
-                h->scratch_bytes = most;
-                if ((rc = dalloc(h, &h->offsets, nk + 1))) return fail(rc);
-                if (!ck(cudaMemcpyAsync(h->offsets, roff.data(), sizeof(int64_t) * (nk + 1), cudaMemcpyHostToDevice, cs), "copy chunk offsets") ||
-                    !ck(cudaMemsetAsync(h->scratch, 0, (size_t)h->scratch_bytes, cs), "clear scratch"))
-                    return fail(ESMF_ERR_CUDA);
-                // each scratch chunk's cost-balanced chunks for the tensor kernel
-                for (size_t c = 0; !by_split && c + 1 < ch.size(); ++c) {
-                    std::vector<BrickDesc> sub(kept.begin() + ch[c], kept.begin() + ch[c + 1]);
-                    const std::vector<int64_t> sp = balance_parts(sub, kChunksPerSM * h->num_sms);
-                    int64_t *dp = nullptr;
-                    if ((rc = dalloc(h, &dp, sp.size()))) return fail(rc);
-                    h->shard_parts.emplace(std::make_pair(ch[c], ch[c + 1]), std::make_pair(dp, (int)sp.size() - 1));
-                    if (!ck(cudaMemcpyAsync(dp, sp.data(), sizeof(int64_t) * sp.size(), cudaMemcpyHostToDevice, cs), "copy chunk parts") ||
-                        !ck(cudaStreamSynchronize(cs), "chunk parts"))
-                        return fail(ESMF_ERR_CUDA);
-                }
-                if (by_split && !ck(cudaStreamSynchronize(cs), "chunk offsets")) return fail(ESMF_ERR_CUDA);
-            }
-        }
         if (use_mode == ESMF_MODE_STORED) {
             if ((rc = dalloc(h, &h->offsets, h->nbricks + 1))) return fail(rc);
             if ((rc = dalloc(h, (unsigned char **)&h->store, (size_t)h->store_bytes))) return fail(rc);
@@ -858,6 +800,65 @@ static int create_impl(const esmf_basis_t *basis, const int32_t *cart, double to
                 !ck(cudaMemcpyAsync(h->pblocks, pblocks_h.data(), sizeof(int) * pblocks_h.size(), cudaMemcpyHostToDevice, cs), "copy pair blocks"))
                 return fail(ESMF_ERR_CUDA);
             if ((rc = launch_pair_table(db, h->pblocks, h->n_ptab, h->prec, h->ptab, s))) return fail(rc);
+        }
+        if (use_mode == ESMF_MODE_DIRECT && h->prec != ESMF_PREC_FP32 && !h->cart) {
+            // integral-direct on the tensor cores: chunks of whole items whose
+            // records fit the scratch buffer (2 GiB, or a quarter of the budget;
+            // an item larger than that is a chunk of its own).  FP64 handles
+            // take it when their budget and memory hold it and the density digits
+            // too, and evaluate in the contraction kernel otherwise.
+            const bool by_split = !is_split16(h->prec);
+            const int eb = elem_bytes(h->prec);
+            int64_t cap = (int64_t)2 << 30;
+            if (budget_bytes > 0) cap = std::min<int64_t>(cap, budget_bytes / 4);
+            const int64_t nk = h->nbricks;
+            std::vector<int64_t> ch{0};
+            int64_t prev = 0;                        // the last item start seen
+            for (int64_t i = 1; i <= nk; ++i) {
+                if (i < nk && !(kept[i].pad & BRICK_ITEM_FIRST)) continue;
+                if ((offs[i] - offs[ch.back()]) * eb > cap && prev > ch.back()) ch.push_back(prev);
+                prev = i;
+            }
+            if (ch.back() != nk) ch.push_back(nk);
+            std::vector<int64_t> roff(nk + 1, 0);
+            int64_t most = 0;
+            for (size_t c = 0; c + 1 < ch.size(); ++c) {
+                for (int64_t i = ch[c]; i < ch[c + 1]; ++i) roff[i] = offs[i] - offs[ch[c]];
+                most = std::max(most, (offs[ch[c + 1]] - offs[ch[c]]) * eb);
+            }
+            bool room = true;
+            if (by_split) {
+                // everything else that the handle keeps is allocated by now
+                const int64_t need = most + (nk + 1) * 8 + (int64_t)split_kbank_bytes(h->nb) +
+                                     (int64_t)split_jbank_bytes(h->nb);
+                room = !h->no_split && (budget_bytes == 0 || h->device_bytes + need <= budget_bytes);
+                if (room && dalloc(h, (unsigned char **)&h->scratch, (size_t)most) != ESMF_OK) {
+                    cudaGetLastError();
+                    room = false;
+                }
+            } else if ((rc = dalloc(h, (unsigned char **)&h->scratch, (size_t)most))) {
+                return fail(rc);
+            }
+            if (room) {
+                h->chunks = ch;
+                h->scratch_bytes = most;
+                if ((rc = dalloc(h, &h->offsets, nk + 1))) return fail(rc);
+                if (!ck(cudaMemcpyAsync(h->offsets, roff.data(), sizeof(int64_t) * (nk + 1), cudaMemcpyHostToDevice, cs), "copy chunk offsets") ||
+                    !ck(cudaMemsetAsync(h->scratch, 0, (size_t)h->scratch_bytes, cs), "clear scratch"))
+                    return fail(ESMF_ERR_CUDA);
+                // each scratch chunk's cost-balanced chunks for the tensor kernel
+                for (size_t c = 0; !by_split && c + 1 < ch.size(); ++c) {
+                    std::vector<BrickDesc> sub(kept.begin() + ch[c], kept.begin() + ch[c + 1]);
+                    const std::vector<int64_t> sp = balance_parts(sub, kChunksPerSM * h->num_sms);
+                    int64_t *dp = nullptr;
+                    if ((rc = dalloc(h, &dp, sp.size()))) return fail(rc);
+                    h->shard_parts.emplace(std::make_pair(ch[c], ch[c + 1]), std::make_pair(dp, (int)sp.size() - 1));
+                    if (!ck(cudaMemcpyAsync(dp, sp.data(), sizeof(int64_t) * sp.size(), cudaMemcpyHostToDevice, cs), "copy chunk parts") ||
+                        !ck(cudaStreamSynchronize(cs), "chunk parts"))
+                        return fail(ESMF_ERR_CUDA);
+                }
+                if (by_split && !ck(cudaStreamSynchronize(cs), "chunk offsets")) return fail(ESMF_ERR_CUDA);
+            }
         }
         if (use_mode == ESMF_MODE_STORED) {
             if (h->cart)

@@ -51,3 +51,23 @@ def test_third_accumulator_does_not_fit(esmf):
             del fill
             torch.cuda.empty_cache()
         close([x[:2].cpu().numpy() for x in (J, K)], ref, 1e-11)
+
+
+def test_direct_budget(esmf):
+    """A direct handle with the scratch buffer stays in its budget, digit tiles included."""
+    import torch
+    w = W.small_random(96, 1, 4, tol=1e-10)
+    D = torch.from_numpy(w.D).cuda()
+    acc = (3 * 96 * 96 + 1) * 8
+    with esmf.FockBuilder(w.basis, w.tol, "direct", "fp64", budget_bytes=1 << 20) as fb:
+        base = fb.stats()
+    assert base["scratch_bytes"] == 0 and base["n_chunks"] == 0
+    taken = 0
+    for extra in range(0, 24 * MB, MB // 4):
+        budget = base["device_bytes"] + extra
+        with esmf.FockBuilder(w.basis, w.tol, "direct", "fp64", budget_bytes=budget) as fb:
+            if fb.stats()["scratch_bytes"]:
+                taken += 1
+                fb.build(D)
+                assert fb.stats()["device_bytes"] <= budget + acc
+    assert taken > 10

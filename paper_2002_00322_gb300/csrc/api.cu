@@ -194,6 +194,7 @@ int dalloc(esmf_fock *h, T **p, size_t count) {
     cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
     if (e != cudaSuccess) {
         *p = nullptr;
+        cudaGetLastError();                 // not for the next launch's check to find
         set_error("cudaMalloc(%zu bytes): %s", count * sizeof(T), cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? ESMF_ERR_OOM : ESMF_ERR_CUDA;
     }
@@ -336,7 +337,6 @@ size_t acc_doubles(const esmf_fock *h, int m) {
 // holds goes back, and the handle's builds take the CUDA-core kernel, which needs
 // none of it.
 void drop_split(esmf_fock *h) {
-    cudaGetLastError();
     dfree(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb));
     dfree(h, (unsigned char **)&h->sjbank, split_jbank_bytes(h->nb));
     if (h->mode == ESMF_MODE_DIRECT) {
@@ -832,17 +832,16 @@ static int create_impl(const esmf_basis_t *basis, const int32_t *cart, double to
                 const int64_t need = most + (nk + 1) * 8 + (int64_t)split_kbank_bytes(h->nb) +
                                      (int64_t)split_jbank_bytes(h->nb);
                 room = !h->no_split && (budget_bytes == 0 || h->device_bytes + need <= budget_bytes);
-                if (room && dalloc(h, (unsigned char **)&h->scratch, (size_t)most) != ESMF_OK) {
-                    cudaGetLastError();
-                    room = false;
-                }
-            } else if ((rc = dalloc(h, (unsigned char **)&h->scratch, (size_t)most))) {
-                return fail(rc);
             }
+            h->scratch_bytes = most;
+            if (room && ((rc = dalloc(h, (unsigned char **)&h->scratch, (size_t)most)) ||
+                         (rc = dalloc(h, &h->offsets, nk + 1)))) {
+                if (!by_split) return fail(rc);
+                room = false;
+            }
+            if (!room) drop_split(h);
             if (room) {
                 h->chunks = ch;
-                h->scratch_bytes = most;
-                if ((rc = dalloc(h, &h->offsets, nk + 1))) return fail(rc);
                 if (!ck(cudaMemcpyAsync(h->offsets, roff.data(), sizeof(int64_t) * (nk + 1), cudaMemcpyHostToDevice, cs), "copy chunk offsets") ||
                     !ck(cudaMemsetAsync(h->scratch, 0, (size_t)h->scratch_bytes, cs), "clear scratch"))
                     return fail(ESMF_ERR_CUDA);

@@ -71,3 +71,33 @@ def test_direct_budget(esmf):
                 fb.build(D)
                 assert fb.stats()["device_bytes"] <= budget + acc
     assert taken > 10
+
+
+def test_create_direct(esmf):
+    """A direct handle is made whenever it fits without the scratch buffer."""
+    import torch
+    w = W.small_random(200, 2, 4, tol=1e-10, edge=10.0, min_dist=1.0)
+    D = torch.from_numpy(w.D).cuda()
+
+    def make():
+        with esmf.FockBuilder(w.basis, w.tol, "direct", "fp64") as fb:
+            return fb.stats()
+    st = make()
+    assert st["scratch_bytes"] > 500 * MB
+    missed = 0
+    for less in (64, 40, 20, 16, 12, 8, 6, 4, 2, 0):
+        fill = hog(st["device_bytes"] + 80 * MB - less * MB)
+        try:
+            missed += make()["scratch_bytes"] == 0
+        finally:
+            del fill
+    for less in range(0, 40, 2):                                  # without the slack of the loop above
+        fill = hog(st["device_bytes"] + 8 * MB - less * MB)
+        try:
+            missed += make()["scratch_bytes"] == 0
+        finally:
+            del fill
+            torch.cuda.empty_cache()
+    assert missed > 0                                             # the fallback ran
+    with esmf.FockBuilder(w.basis, 1e-4, "direct", "fp64") as fb:
+        assert fb.device_error() == 0 and torch.isfinite(fb.build(D)[0]).all()

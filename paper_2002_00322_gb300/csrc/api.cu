@@ -348,6 +348,17 @@ void drop_split(esmf_fock *h) {
     h->no_split = true;
 }
 
+// dalloc for memory that a build cannot do without: where it does not fit, the
+// memory of the digit-splitting path goes back first
+template <typename T>
+int dneed(esmf_fock *h, T **p, size_t count) {
+    const int rc = dalloc(h, p, count);
+    if (rc != ESMF_ERR_OOM) return rc;
+    if (!split_path(h) || !(h->skbank || h->scratch)) return rc;
+    drop_split(h);
+    return dalloc(h, p, count);
+}
+
 int ensure_work(esmf_fock *h, int m) {
     if (split_path(h) && !h->skbank &&
         (dalloc(h, (unsigned char **)&h->skbank, split_kbank_bytes(h->nb)) != ESMF_OK ||
@@ -360,8 +371,8 @@ int ensure_work(esmf_fock *h, int m) {
         RET(dalloc(h, &h->sched, 1));
     }
     if (h->tol_d > 0.0 && !h->dw) {
-        RET(dalloc(h, &h->dw, (size_t)h->np * h->np));
-        RET(dalloc(h, &h->dwb, (size_t)h->nb * h->nb));
+        RET(dneed(h, &h->dw, (size_t)h->np * h->np));
+        RET(dneed(h, &h->dwb, (size_t)h->nb * h->nb));
     }
     if (m <= h->work_m) return ESMF_OK;
     const size_t tb = density_typed_bytes(h->prec);
@@ -372,7 +383,7 @@ int ensure_work(esmf_fock *h, int m) {
     if (split_path(h) && dalloc(h, &h->acc, acc_doubles(h, m)) != ESMF_OK) drop_split(h);
     if (!h->acc) RET(dalloc(h, &h->acc, acc_doubles(h, m)));
     h->acc_n = acc_doubles(h, m);
-    if (tb) RET(dalloc(h, (unsigned char **)&h->Dt, (size_t)m * h->n * h->n * tb));
+    if (tb) RET(dneed(h, (unsigned char **)&h->Dt, (size_t)m * h->n * h->n * tb));
     h->work_m = m;
     return ESMF_OK;
 }
@@ -1571,7 +1582,7 @@ int esmf_energy_gradient(esmf_fock_t *h, int n_occ, double c0, const double *G, 
     if (need > h->ework_n) {
         dfree(h, &h->ework, h->ework_n);
         h->ework_n = 0;
-        RET(dalloc(h, &h->ework, need));
+        RET(dneed(h, &h->ework, need));
         h->ework_n = need;
     }
     const EnergyWork w = energy_work_layout(h->ework, n, n_occ);
@@ -1612,7 +1623,7 @@ int esmf_gvp_gradient(esmf_fock_t *h, int n_occ, double c0, const double *G, con
     if (need > h->ework_n) {
         dfree(h, &h->ework, h->ework_n);
         h->ework_n = 0;
-        RET(dalloc(h, &h->ework, need));
+        RET(dneed(h, &h->ework, need));
         h->ework_n = need;
     }
     const EnergyWork w = energy_work_layout(h->ework, n, n_occ);
@@ -1673,8 +1684,8 @@ int esmf_fock_build_host(esmf_fock_t *h, int m, const double *D_host, double *J_
         dfree(h, &h->sK, (size_t)h->stage_m * mat); dfree(h, &h->sF, (size_t)h->stage_m * mat);
         dfree(h, &h->st, (size_t)h->stage_m);
         h->stage_m = 0;
-        RET(dalloc(h, &h->sD, m * mat)); RET(dalloc(h, &h->sJ, m * mat)); RET(dalloc(h, &h->sK, m * mat));
-        RET(dalloc(h, &h->sF, m * mat)); RET(dalloc(h, &h->st, (size_t)m));
+        RET(dneed(h, &h->sD, m * mat)); RET(dneed(h, &h->sJ, m * mat)); RET(dneed(h, &h->sK, m * mat));
+        RET(dneed(h, &h->sF, m * mat)); RET(dneed(h, &h->st, (size_t)m));
         h->stage_m = m;
     }
     cudaStream_t s = (cudaStream_t)stream;

@@ -101,3 +101,24 @@ def test_create_direct(esmf):
     assert missed > 0                                             # the fallback ran
     with esmf.FockBuilder(w.basis, 1e-4, "direct", "fp64") as fb:
         assert fb.device_error() == 0 and torch.isfinite(fb.build(D)[0]).all()
+
+
+def test_staging_of_host_buffers_does_not_fit(esmf):
+    """Memory that a build cannot do without takes the digit tiles' place."""
+    import torch
+    n, m = 800, 16
+    w = W.small_random(n, 1, 3, tol=1e-6, edge=400.0)
+    D = torch.randn((m, n, n), dtype=torch.float64, generator=torch.Generator().manual_seed(1)).pin_memory()
+    pin = lambda: torch.empty((m, n, n), dtype=torch.float64).pin_memory()  # noqa: E731
+    with esmf.FockBuilder(w.basis, w.tol, "stored", "fp64") as fb:
+        ref = [x.numpy() for x in fb.build_host(D, pin(), pin())[:2]]
+    with esmf.FockBuilder(w.basis, w.tol, "stored", "fp64") as fb:
+        one = torch.zeros((1, n, n), dtype=torch.float64, device="cuda")
+        fb.build(one)
+        fill = hog(4 * m * n * n * 8 - 64 * MB)                   # less than the staging alone
+        try:
+            got = [x.numpy() for x in fb.build_host(D, pin(), pin())[:2]]
+        finally:
+            del fill
+            torch.cuda.empty_cache()
+        close(got, ref, 1e-11)

@@ -348,14 +348,27 @@ void drop_split(esmf_fock *h) {
     h->no_split = true;
 }
 
+// The same for the exchange of a density-fitted FP64 handle with density tiles
+// for mt densities: build_df then lays the factor out for cuBLAS.
+void drop_df_split(esmf_fock *h, int mt) {
+    const size_t tb = df_split_tile_bytes(h->n, h->naux), ldD = (size_t)((h->n + 63) / 64) * 64;
+    dfree(h, &h->dfTiles, tb);
+    dfree(h, &h->dfYt, tb * h->df_group);
+    dfree(h, &h->dfS, df_split_sum_bytes(h->n, h->df_group));
+    dfree(h, &h->dfDtl, df_split_tile_bytes(h->n, mt));
+    dfree(h, &h->dfeD, mt * ldD);
+    dfree(h, &h->dfED, 2 * (size_t)mt);
+}
+
 // dalloc for memory that a build cannot do without: where it does not fit, the
-// memory of the digit-splitting path goes back first
+// memory of the digit-splitting paths goes back first
 template <typename T>
 int dneed(esmf_fock *h, T **p, size_t count) {
     const int rc = dalloc(h, p, count);
     if (rc != ESMF_ERR_OOM) return rc;
-    if (!split_path(h) || !(h->skbank || h->scratch)) return rc;
-    drop_split(h);
+    if (h->mode == ESMF_MODE_DF && h->dfTiles) drop_df_split(h, h->df_m);
+    else if (split_path(h) && (h->skbank || h->scratch)) drop_split(h);
+    else return rc;
     return dalloc(h, p, count);
 }
 
@@ -1288,25 +1301,31 @@ int build_df(esmf_fock_t *h, int m, const double *D, double *J, double *K, doubl
     const size_t nn = (size_t)h->n * h->n;
     const size_t ldD = (size_t)((h->n + 63) / 64) * 64;
     if (m > h->df_m) {
-        if (h->dfTiles) {
-            dfree(h, &h->dfDtl, df_split_tile_bytes(h->n, h->df_m));
-            dfree(h, &h->dfeD, h->df_m * ldD);
-            dfree(h, &h->dfED, 2 * (size_t)h->df_m);
-        }
-        dfree(h, (unsigned char **)&h->dfDt, es == 4 ? h->df_m * nn * es : 1);
-        dfree(h, (unsigned char **)&h->dfJt, h->df_m * nn * es);
-        dfree(h, (unsigned char **)&h->dfKt, h->df_m * nn * es); dfree(h, (unsigned char **)&h->dfg, (size_t)h->df_m * h->naux * es);
+        const size_t o = (size_t)h->df_m;
+        dfree(h, &h->dfDtl, df_split_tile_bytes(h->n, h->df_m));
+        dfree(h, &h->dfeD, o * ldD);
+        dfree(h, &h->dfED, 2 * o);
+        dfree(h, (unsigned char **)&h->dfDt, es == 4 ? o * nn * es : 1);
+        dfree(h, (unsigned char **)&h->dfJt, o * nn * es);
+        dfree(h, (unsigned char **)&h->dfKt, o * nn * es);
+        dfree(h, (unsigned char **)&h->dfg, o * h->naux * es);
         h->df_m = 0;
-        RET(dalloc(h, (unsigned char **)&h->dfDt, es == 4 ? m * nn * es : 1));
-        RET(dalloc(h, (unsigned char **)&h->dfJt, m * nn * es));
-        RET(dalloc(h, (unsigned char **)&h->dfKt, m * nn * es));
-        RET(dalloc(h, (unsigned char **)&h->dfg, (size_t)m * h->naux * es));
-        if (h->dfTiles) {
-            RET(dalloc(h, &h->dfDtl, df_split_tile_bytes(h->n, m)));
-            RET(dalloc(h, &h->dfeD, m * ldD));
-            RET(dalloc(h, &h->dfED, 2 * (size_t)m));
-        }
+        RET(dneed(h, (unsigned char **)&h->dfDt, es == 4 ? m * nn * es : 1));
+        RET(dneed(h, (unsigned char **)&h->dfJt, m * nn * es));
+        RET(dneed(h, (unsigned char **)&h->dfKt, m * nn * es));
+        RET(dneed(h, (unsigned char **)&h->dfg, (size_t)m * h->naux * es));
+        if (h->dfTiles && (dalloc(h, &h->dfDtl, df_split_tile_bytes(h->n, m)) != ESMF_OK ||
+                           dalloc(h, &h->dfeD, m * ldD) != ESMF_OK || dalloc(h, &h->dfED, 2 * (size_t)m) != ESMF_OK))
+            drop_df_split(h, m);
         h->df_m = m;
+    }
+    if (es == 8 && !h->dfTiles && !h->dfY) {
+        // the exchange by digit splitting was given up: cuBLAS' second layout of the factor
+        if (!h->dfB2) RET(dalloc(h, (unsigned char **)&h->dfB2, h->naux * nn * es));
+        RET(dalloc(h, (unsigned char **)&h->dfY, h->naux * nn * es));
+        RET(launch_df_layouts(h->naux, h->n, (const double *)h->dfB, 0, nullptr, h->dfB2, s));
+        CKR(cudaStreamSynchronize(s));           // builds on other streams read it too
+        h->store_bytes = (int64_t)(2 * h->naux * nn * es);
     }
     DfSplit sp;
     if (h->dfTiles) {

@@ -122,3 +122,30 @@ def test_staging_of_host_buffers_does_not_fit(esmf):
             del fill
             torch.cuda.empty_cache()
         close(got, ref, 1e-11)
+
+
+def test_density_tiles_do_not_fit(esmf):
+    """A density-fitted handle goes back to cuBLAS when the tiles of many densities do not fit."""
+    import torch
+    n, m = 130, 512
+    w = W.small_random(n, 1, 6, edge=12.0, min_dist=1.0)
+    aux = W.even_tempered_aux(w.basis, count=2)
+    D = torch.randn((m, n, n), dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(2))
+    J, K = torch.empty_like(D), torch.empty_like(D)
+    with esmf.FockBuilder(w.basis, 0.0, "df", "fp64", aux=aux) as fb:
+        ref = [x.cpu().numpy() for x in fb.build(D[:2])[:2]]
+        fb.build(D, J, K, want_traces=False)                      # loads cuBLAS' kernels for these sizes
+    with esmf.FockBuilder(w.basis, 0.0, "df", "fp64", aux=aux) as fb:
+        fb.build(D[:1])
+        tiles = m * 6 * 114688                                    # 128 x 64 tiles of 112 KB, two by three a density
+        fill = hog(tiles - 16 * MB)
+        try:
+            fb.build(D, J, K, want_traces=False)
+            st = fb.stats()["store_bytes"]
+        finally:
+            del fill
+            torch.cuda.empty_cache()
+        assert st == 2 * len(aux[1]) * n * n * 8
+        close([x[:2].cpu().numpy() for x in (J, K)], ref, 1e-12)
+        fb.build(D, J, K, want_traces=False)
+        close([x[:2].cpu().numpy() for x in (J, K)], ref, 1e-12)

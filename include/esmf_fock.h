@@ -394,7 +394,9 @@ int esmf_fock_set_path(esmf_fock_t *h, int path);
  * FP32, 8/4 for FP64) as the median of `reps` builds (after one warm-up) on
  * the caller's device buffers D (read), J and K (overwritten), and records
  * the fastest; later builds with the same m use it.  *chosen (optional)
- * receives it.  Synchronises the stream.  Errors: as esmf_fock_build.
+ * receives it.  FP64 and F32X2 builds on the tensor cores always pass over up
+ * to 16 densities: one build, *chosen = 16, nothing recorded.  Synchronises the
+ * stream.  Errors: as esmf_fock_build.
  */
 int esmf_fock_autotune(esmf_fock_t *h, int m, const double *D, double *J, double *K, int reps,
                        void *stream, int *chosen);

@@ -1767,6 +1767,16 @@ int esmf_fock_autotune(esmf_fock_t *h, int m, const double *D, double *J, double
     if (!g.ok) { set_error("cudaSetDevice failed"); return ESMF_ERR_CUDA; }
     const bool tensor = (h->mode == ESMF_MODE_STORED || tensor_direct(h)) && is_split16(h->prec) &&
                         h->path != ESMF_PATH_CUDA_CORE;
+    if (split_path(h) && h->path != ESMF_PATH_CUDA_CORE && h->tol_d == 0.0) {
+        // the splitting kernel's passes take 16 densities whatever is asked for, and a
+        // choice timed on it would go to the CUDA-core kernel
+        RET(esmf_fock_build(h, m, D, J, K, nullptr, nullptr, stream));
+        if (split_path(h)) {
+            CKR(cudaStreamSynchronize((cudaStream_t)stream));
+            if (chosen) *chosen = 16;
+            return ESMF_OK;
+        }
+    }
     std::vector<int> cand;
     if (tensor) { cand.push_back(16); if (m > 8) cand.push_back(8); }
     else if (h->prec == ESMF_PREC_FP64 || h->prec == ESMF_PREC_F32X2) { cand.push_back(8); cand.push_back(4); }

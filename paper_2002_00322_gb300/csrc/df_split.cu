@@ -66,11 +66,9 @@ constexpr int DF_SMEM = OFF_CTRL + 1024;
 constexpr int EPI_WARPS = 16;
 constexpr int DF_THREADS = 64 + 32 * EPI_WARPS;
 constexpr int EMIN = 1022 - 600;              // smallest exponent field of a row
-constexpr int DMIN = -500, DMAX = 500;        // exponents of the densities that digits serve
 constexpr int BMAX = 250;                     // largest exponent of the factor
 constexpr unsigned long long SL_MASK = (1ull << 36) - 1;   // SL below 2^36 SH
 constexpr int MAX_BLOCKS = 2048;              // blocks of 64 summed elements that SL and SH hold
-constexpr uint32_t POLLS = 1u << 22;
 
 struct DfCtrl {
     uint64_t full[STAGES], empty[STAGES], accfull, accfree;
@@ -78,10 +76,6 @@ struct DfCtrl {
     int abort_flag, never;
 };
 static_assert(sizeof(DfCtrl) <= 1024 && DF_SMEM <= 227 * 1024, "shared memory");
-
-__device__ __forceinline__ bool wait_for(uint64_t *bar, uint32_t parity, const volatile int *abort) {
-    return mbar_wait(bar, parity, abort, POLLS);
-}
 
 // 32 lanes x 32-bit, 4 consecutive columns per thread
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float *v) {
@@ -95,11 +89,6 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float *v) {
 
 // exponent field of x: |x| < 2^(field - 1022)
 __device__ __forceinline__ int exp_field(double x) { return (int)(((uint32_t)__double2hiint(x) >> 20) & 0x7ffu); }
-
-// a density whose largest exponent field is `top` and not served by digits
-__device__ __forceinline__ bool beyond_digits(int top) {
-    return top != 0 && (top > 1022 + DMAX || top <= 1022 + DMIN);
-}
 
 // digits of eight fixed-point values as the eight-element pieces of a tile's
 // group: digit i at dst + i * 2048 (dst addresses the row)
@@ -187,7 +176,7 @@ __global__ void k_df_dcols(const double *D, int n, int ldD, int16_t *eD, int *ED
         for (int r = 0; r < n; ++r) {
             const double v = D[((int64_t)k * n + r) * n + s];
             q = fma(v, v, q);
-            e = max(e, v != 0.0 ? max(exp_field(v), 1) : 0);
+            e = max(e, field_of(v));
         }
     eD[(int64_t)k * ldD + s] = (int16_t)(max(e, EMIN) - 1022);
     if (e == 0) return;

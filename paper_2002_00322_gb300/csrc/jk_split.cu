@@ -95,7 +95,7 @@ constexpr int split_threads = 64 + CONV_THREADS + 32 * epi_warps<MP>;
 // leaves FP64's normal range.  Neither is seen beside the handle's largest
 // integrals, which are above 2^-260 (a basis' exponents have squares in FP64's
 // range), and the densities' largest elements, above 2^DMIN.
-constexpr int EMIN_V = 1022 - 300, EMIN_D = 1022 - 640, DMIN = -500, DMAX = 500;
+constexpr int EMIN_V = 1022 - 300, EMIN_D = 1022 - 640;
 constexpr int REGION = 256;                       // tensor-memory columns per view buffer
 static_assert(OFF_RING % 1024 == 0 && OFF_REC % 16 == 0, "operand tiles");
 static_assert(NT * 2 * MPM <= REGION, "view region");
@@ -115,12 +115,6 @@ struct SplitCtrl {
     uint16_t vpos[512];
 };
 static_assert(SPLIT_SMEM <= 227 * 1024 && sizeof(SplitCtrl) <= CTRL_BYTES, "control block");
-
-// Polls after which a wait gives up (every wait here is far shorter).
-constexpr uint32_t POLLS = 1u << 22;
-__device__ __forceinline__ bool wait_for(uint64_t *bar, uint32_t parity, const volatile int *abort) {
-    return mbar_wait(bar, parity, abort, POLLS);
-}
 
 // Views of a brick in the order they run: 0-3 exchange V1..V4, 4 Coulomb J1, 5
 // Coulomb J2 (see jk_umma.cu); the next one after v that the brick has.
@@ -164,16 +158,6 @@ __device__ __forceinline__ void tmem_ld_half4(uint32_t taddr, float *v) {
                  : "r"(taddr));
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// a density whose largest exponent field is `top` and not served by digits
-__device__ __forceinline__ bool beyond_digits(int top) {
-    return top != 0 && (top > 1022 + DMAX || top <= 1022 + DMIN);
-}
-// exponent field of x, 1 for subnormal numbers, 0 for zero
-__device__ __forceinline__ int field_of(double x) {
-    const int f = (__double2hiint(x) >> 20) & 0x7ff;
-    return x != 0.0 ? max(f, 1) : 0;
 }
 
 // canonical K-major operand tile: row n (density column of the MMA), k = b*8 + d

@@ -7,8 +7,29 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "umma.cuh"
+
 namespace esmf {
 namespace split {
+
+// Polls after which a wait of these kernels gives up (every wait is far shorter).
+constexpr uint32_t POLLS = 1u << 22;
+__device__ __forceinline__ bool wait_for(uint64_t *bar, uint32_t parity, const volatile int *abort) {
+    return umma::mbar_wait(bar, parity, abort, POLLS);
+}
+
+// ---- densities that digits serve: the largest element in [2^DMIN, 2^DMAX), where
+// the exponents of all products and the squares behind norms stay in FP64's
+// range; top is a density's largest exponent field, 0 for a zero one
+constexpr int DMIN = -500, DMAX = 500;
+__device__ __forceinline__ bool beyond_digits(int top) {
+    return top != 0 && (top > 1022 + DMAX || top <= 1022 + DMIN);
+}
+// exponent field of x, 1 for subnormal numbers, 0 for zero: |x| < 2^(field - 1022)
+__device__ __forceinline__ int field_of(double x) {
+    const int f = (__double2hiint(x) >> 20) & 0x7ff;
+    return x != 0.0 ? max(f, 1) : 0;
+}
 
 // ---- digits.  x 2^(BITS - e) rounded to an integer of magnitude at most
 // 2^BITS, for |x| < 2^e, e = emax - 1022 with emax the largest exponent field

@@ -104,8 +104,9 @@ typedef struct {
     double  create_ms;          /* wall time of esmf_fock_create               */
     int32_t screening;          /* ESMF_SCREEN_*                               */
     int64_t n_pairs_kept;       /* pairs in at least one kept quartet          */
-    int64_t n_chunks;           /* integral-direct FP16X2/BF16X2: chunks each  */
-                                /* build regenerates (0 otherwise)             */
+    int64_t n_chunks;           /* integral-direct FP64/FP16X2/BF16X2 with a   */
+                                /* scratch buffer: chunks each build           */
+                                /* regenerates (0 otherwise)                   */
     int64_t scratch_bytes;      /* their scratch buffer (part of device_bytes) */
 } esmf_stats_t;
 
@@ -375,13 +376,26 @@ int esmf_fock_set_density_screening(esmf_fock_t *h, double tol_d);
 
 /*
  * Contraction kernel choice for stored FP64, F32X2, FP16X2 and BF16X2
- * integrals: ESMF_PATH_AUTO uses the tensor-core kernels (for FP64 and F32X2
- * by error-free splitting, as accurate as FP64 arithmetic),
+ * integrals: ESMF_PATH_AUTO uses the tensor-core kernels,
  * ESMF_PATH_CUDA_CORE the CUDA-core kernels (same results within rounding;
- * kept as a cross-check).  Integral-direct FP64 handles of s bases take the
- * splitting kernel from a scratch buffer of integral records (at most 2 GiB, or
- * a quarter of the budget) when it and the density digits fit the budget.  FP32
- * handles always use the CUDA-core kernels.  Errors: INVALID_ARG.
+ * kept as a cross-check, and for outputs that need their own accuracy).
+ * The tensor-core kernel of FP64 and F32X2 works on digits in fixed point: a
+ * product V D is off by at most 2^-53 |V| Db + 2^-58 Vb Db, with Vb the largest
+ * integral of its 8x8x8x8 block and Db the largest density of its 8x8 block.  J
+ * and K as a whole are as accurate as in FP64 arithmetic; single elements that only
+ * much smaller products feed (J of functions that hardly overlap, or densities
+ * that differ by many decades within a block) are so on ESMF_PATH_CUDA_CORE only.
+ * Densities whose largest element is not in [2^-500, 2^500), infinities and NaN
+ * take FP64 arithmetic (and the others of their pass with them).
+ * Density-fitted K in FP64 has the same kind of bound (relative to the rows of
+ * the fitted factor and the columns of D) and no other path.
+ * Integral-direct FP64 handles of s bases take the splitting kernel from a
+ * scratch buffer of integral records (at most 2 GiB, or a quarter of the budget)
+ * when it and the density digits fit the budget and memory.  FP32 handles always
+ * use the CUDA-core kernels: half the FP64 store's memory, but a stored FP64 build
+ * is faster (200 functions, 16 densities: 2.8 ms against 4.1).  So do builds with
+ * density-weighted screening, in every precision (FP64: 55 ms there when nothing
+ * is screened).  Errors: INVALID_ARG.
  */
 #define ESMF_PATH_AUTO       0
 #define ESMF_PATH_CUDA_CORE  1

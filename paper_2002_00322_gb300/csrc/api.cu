@@ -1034,7 +1034,10 @@ int esmf_fock_create_df(const esmf_basis_t *basis, const esmf_aux_t *aux, int pr
     if (es == 8) {
         // digit tiles of the factor and of Y for as many densities per pass as fit
         // 2.5 GiB; without room for them, or with a factor that the digits cannot
-        // hold, the exchange stays on cuBLAS
+        // hold, the exchange stays on cuBLAS.  The size hardly matters beyond filling
+        // the SMs (16 densities, 0.65 / 1.3 / 2.0 / 2.7 / 5.2 / 10.4 GB: 120 functions
+        // 3.05 / 2.99 / 2.75 / 2.74 / 2.75 / 2.75 ms, 200 functions 24.5 / 23.9 / 25.6 /
+        // 23.6 / 25.2 / 25.1, 300 functions 91.5 up to 2.7 GB, 89.9, 87.1).
         std::vector<int16_t> rows(n);
         if ((rc = dalloc(h, &h->dfeB, 2 * (size_t)n))) return fail(rc);
         if ((rc = launch_df_split_rows(B, naux, n, h->dfeB, h->dfeB + n, cs))) return fail(rc);

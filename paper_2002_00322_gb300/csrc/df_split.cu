@@ -1,5 +1,5 @@
-// Density-fitted exchange in FP64 accuracy on the sm_103a tensor cores, by the
-// error-free digit splitting of jk_split.cu:
+// Density-fitted exchange in FP64 on the sm_103a tensor cores, by the digit
+// splitting of jk_split.cu:
 //   Y_k[P][p][s] = sum_r B[P][p][r] D_k[r][s],   K_k[p][q] = sum_{P,s} Y_k[P][p][s] B[P][q][s]
 // (GB300's FP64 pipe runs two FMA per clock and SM, so cuBLAS DGEMMs of the two
 // products took 426 of the 430 ms of a 16-density build over 200 functions and
@@ -29,7 +29,9 @@
 // (df_ranges).  The digit pairs left out weigh 2^-63 of that product each.  A row
 // spans all auxiliaries, whose elements differ by decades: with six digits and
 // t < 6 the error of K against 64-bit references was 5e-13 over 200 functions
-// (DGEMM 3.9e-14).
+// (DGEMM 3.9e-14).  The bound is normwise: an element of B 2^-k of its row's
+// largest over all auxiliaries keeps 63 - k bits, one of D likewise in its column,
+// and Y is rounded to 2^-62 of its bound, which all columns share.
 //
 // Digits serve densities whose largest element lies in [2^-500, 2^500), where
 // the squares behind the bound on Y stay in FP64's range; k_df_plain takes the

@@ -1,26 +1,35 @@
-// FP64-accurate grouped J/K contraction on the sm_103a tensor cores (tcgen05)
-// for FP64 and double-FP32 integral stores: every operand is split without
-// error into fixed-point digits that the FP16 tensor pipe multiplies and sums
-// exactly (the error-free splitting of Ozaki, Ogita, Oishi and Rump 2012, in
-// its fixed-point form).
+// FP64 grouped J/K contraction on the sm_103a tensor cores (tcgen05) for FP64 and
+// double-FP32 integral stores: every operand is rounded to a fixed-point number
+// relative to its block's largest element, whose digits the FP16 tensor pipe
+// multiplies and sums exactly (the splitting of Ozaki, Ogita, Oishi and Rump 2012,
+// in its fixed-point form).
 //
 // A brick (P Q | R S) feeds the six GEMM views of jk_umma.cu (64 output rows,
 // 64 terms, all densities as columns).  With one power of two 2^eV per brick
 // and one 2^eD per density and 8 x 8 density block,
 //   V = 2^(eV-8) sum_i x_i 2^(-9 i), i < 7,   D = 2^(eD-8) sum_j y_j 2^(-9 j), j < 6
 // where the digits x_i, y_j are integers in [-256, 256], exact in FP16: 63 bits
-// below the brick's largest integral, 54 below the block's largest density (an
-// FP64 significand has 53).  The integrals have a digit more because a brick's
-// span decades while a block's densities mostly do not: with six digits the
-// rounding of the small ones made the whole error larger than FP64
-// arithmetic's (relative to 64-bit references, 24 functions: K 7.0e-16 against
-// 5.2e-16; with seven 4.9e-16).  Then
+// below the brick's largest integral, 54 below the block's largest density.  The
+// integrals have a digit more because a brick's span decades while a block's
+// densities mostly do not (with six digits K of 24 functions was further from
+// 64-bit references than FP64 arithmetic's, 7.0e-16 against 5.2e-16).  Then
 //   V . D = 2^(eV+eD-16) sum_t 2^(-9 t) c_t,   c_t = sum_{i+j=t} x_i . y_j
 // and each c_t is an integer that FP32 accumulation in tensor memory holds
 // exactly: 64 terms of at most 2^16 per digit pair, below 2^24 for t <= 3; a
 // last place rounded in a later t weighs less than 2^-51 of the largest
 // product.  All digit pairs with t <= 6 are formed; the others are below 2^-60
 // of the largest product.
+//
+// Accuracy: with Vb the largest integral of a brick and Db the largest density of
+// an 8 x 8 block, each product V D of a sum is off by at most 2^-53 |V| Db +
+// 2^-58 Vb Db, and every brick sum is rounded once.  In the norm of J or K that is
+// less than FP64 arithmetic's rounding: against 113-bit sums, means over eight
+// molecules of 24 functions, J 4.1e-16 and K 3.8e-16 (k_jk_cuda<double> 5.1e-16 and
+// 4.6e-16), three of 40 functions 3.7e-16 and 3.9e-16 (4.4e-16 and 4.7e-16).  Single
+// outputs that only products far below Vb Db feed keep fewer digits than there: J of
+// functions that hardly overlap (products below 2^-58) none.  (Scaling the Coulomb operands by the
+// Schwarz bounds kept those, but digits of their own for W cost 16 % of a build of
+// 200 functions and raised the error of J in the norm to 5.4e-16.)
 //
 // MMA N covers the digits: with the density digits of a block as consecutive
 // operand rows [y_0 | y_1 | ...], the digit x_i multiplies a run of them at

@@ -124,6 +124,7 @@ struct esmf_fock {
     // range, or no memory for the tiles)
     void *skbank = nullptr, *sjbank = nullptr;
     bool no_split = false;
+    bool captured = false;         // a build went into a CUDA graph, which holds the addresses of work memory
     void *Dt = nullptr;            // D in the CUDA-core arithmetic type (FP32 / double-FP32), work_m densities
     double *ework = nullptr;       // ESMF energy / gradient work memory
     size_t ework_n = 0;
@@ -361,11 +362,12 @@ void drop_df_split(esmf_fock *h, int mt) {
 }
 
 // dalloc for memory that a build cannot do without: where it does not fit, the
-// memory of the digit-splitting paths goes back first
+// memory of the digit-splitting paths goes back first, unless a captured graph
+// may still use it
 template <typename T>
 int dneed(esmf_fock *h, T **p, size_t count) {
     const int rc = dalloc(h, p, count);
-    if (rc != ESMF_ERR_OOM) return rc;
+    if (rc != ESMF_ERR_OOM || h->captured) return rc;
     if (h->mode == ESMF_MODE_DF && h->dfTiles) drop_df_split(h, h->df_m);
     else if (split_path(h) && (h->skbank || h->scratch)) drop_split(h);
     else return rc;
@@ -1371,6 +1373,11 @@ int build_range(esmf_fock_t *h, int64_t b0, int64_t b1, int m, const double *D, 
         (traces && !is_device_ptr(traces))) {
         set_error("D, J, K, F and traces must be device memory");
         return ESMF_ERR_INVALID_ARG;
+    }
+    if (stream && !h->captured) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing((cudaStream_t)stream, &st) != cudaSuccess) cudaGetLastError();
+        h->captured = st != cudaStreamCaptureStatusNone;
     }
     if (h->mode == ESMF_MODE_DF) {
         if (b0 != 0 || b1 != h->nbricks) { set_error("density-fitted handles build whole only"); return ESMF_ERR_UNSUPPORTED; }

@@ -149,3 +149,34 @@ def test_density_tiles_do_not_fit(esmf):
         close([x[:2].cpu().numpy() for x in (J, K)], ref, 1e-12)
         fb.build(D, J, K, want_traces=False)
         close([x[:2].cpu().numpy() for x in (J, K)], ref, 1e-12)
+
+
+def test_captured_builds_keep_their_memory(esmf):
+    """A graph replays over the memory that it was captured with: none of it goes back for another call."""
+    import torch
+    n, m = 800, 16
+    w = W.small_random(n, 1, 3, tol=1e-6, edge=400.0)
+    D = torch.randn((m, n, n), dtype=torch.float64, generator=torch.Generator().manual_seed(1)).pin_memory()
+    J, K = torch.empty_like(D).pin_memory(), torch.empty_like(D).pin_memory()
+    with esmf.FockBuilder(w.basis, w.tol, "stored", "fp64") as fb:
+        one = D[:1].cuda()
+        Jd, Kd = torch.empty_like(one), torch.empty_like(one)
+        fb.build(one, Jd, Kd, want_traces=False)
+        ref = [x.cpu().numpy() for x in (Jd, Kd)]
+        graph = torch.cuda.CUDAGraph()
+        stream = torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+            fb.build(one, Jd, Kd, want_traces=False, stream=stream)
+        used = fb.stats()["device_bytes"]
+        fill = hog(4 * m * n * n * 8 - 64 * MB)
+        try:
+            with pytest.raises(esmf.EsmfError, match="out of memory"):
+                fb.build_host(D, J, K)
+        finally:
+            del fill
+            torch.cuda.empty_cache()
+        assert fb.stats()["device_bytes"] >= used
+        Jd.zero_(), Kd.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        close([x.cpu().numpy() for x in (Jd, Kd)], ref, 1e-11)

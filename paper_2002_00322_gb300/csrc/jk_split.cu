@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(256) k_split_dbank(const double *D, int n, int
         t[h] = in ? Dk[(int64_t)(q + h) * n + p] : 0.0;
     }
     const int f = __reduce_max_sync(0xffffffffu, max(field_of(v[0]), field_of(v[1])));
-    if (lane == 0 && live && f > top[kk]) atomicMax(top + kk, f);
+    if (lane == 0 && live && f) atomicMax(top + kk, f);
     auto emit = [&](const double *x, unsigned char *base, int row, int rows, int16_t *eout) {
         const uint32_t h0 = (uint32_t)__double2hiint(x[0]), h1 = (uint32_t)__double2hiint(x[1]);
         int e = max((int)((h0 >> 20) & 0x7ffu), (int)((h1 >> 20) & 0x7ffu));

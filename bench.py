@@ -139,7 +139,8 @@ def stored_roofline(prec, st, m, n, kern_s, alu_peaks, workload="stored_n200_m16
     flops = st["n_quartets_kept"] * 20 * m
     ach = 27 * flops / kern_s / 1e12
     return {"bound": "tensor", "achieved": round(ach, 3), "peak": pk, "unit": "TFLOP/s", "frac": round(ach / pk, 4),
-            "traffic": None, "peak_source": f"{src} 16-bit tensor rate; 27 digit products per FP64 product",
+            "traffic": ncu_traffic("k_jk_split", prec, workload),
+            "peak_source": f"{src} 16-bit tensor rate; 27 digit products per FP64 product",
             "kernel": "k_jk_split", "kernel_ms": round(kern_s * 1e3, 4), "algorithmic_flops": flops}
 
 

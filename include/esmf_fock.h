@@ -443,10 +443,10 @@ int esmf_fock_kernel_time(esmf_fock_t *h, double *ms, int64_t *launches, int res
  * synchronise the device and stall unrelated streams.  The paper has no
  * counterpart; it is a property of this library's memory handling only.
  *
- * Same arguments and asynchrony as esmf_fock_build.  Stored FP64 and FP32
- * handles and integral-direct handles run the same CUDA-core kernels as
- * esmf_fock_build (with the handle's autotuned densities per pass), so the
- * results are the same.  Handles with split 16-bit stores (FP16X2 / BF16X2)
+ * Same arguments and asynchrony as esmf_fock_build.  Stored FP64, F32X2 and FP32
+ * handles and integral-direct handles run the CUDA-core kernels (with the
+ * handle's autotuned densities per pass): those of esmf_fock_build for FP32, of
+ * its ESMF_PATH_CUDA_CORE for FP64 and F32X2.  Handles with split 16-bit stores (FP16X2 / BF16X2)
  * run the CUDA-core kernel over that store here, not the tensor-core kernel
  * (which needs per-handle density tiles in work memory): their results equal
  * esmf_fock_build's within the precision's tolerance (2e-6 relative for

@@ -40,7 +40,8 @@
 //
 // What bounds it: the MMAs (3.6K cycles per block of full size) and the
 // tensor-memory reads after each block (448 of the 512 columns are one
-// accumulator, so they do not overlap).  Sixteen warps read, a quarter of the
+// accumulator, so they do not overlap): at 120 functions the tensor pipe is busy 32
+// and 41 % of the two products, the ALU 41 and 16 %.  Sixteen warps read, a quarter of the
 // columns each (c_0 past the conversion unit): 200 functions, 700 auxiliaries, 16
 // densities 26.1 -> 23.7 ms against eight.
 //

@@ -5,8 +5,9 @@
 // framework or a serving process with a fixed memory plan), and latency-bound
 // loops where a cudaMalloc/cudaFree pair would synchronise the device and
 // stall other streams.  esmf_fock_build_noalloc serves them: for stored FP64
-// and FP32 handles and integral-direct handles it runs the same CUDA-core
-// contraction and finalisation kernels as esmf_fock_build; for split 16-bit
+// and FP32 handles and integral-direct handles it runs the CUDA-core
+// contraction and finalisation kernels (in FP64 those of ESMF_PATH_CUDA_CORE:
+// the digit-splitting kernel needs tiles in handle work memory); for split 16-bit
 // stores it runs the CUDA-core kernel over the store (the tensor-core kernel
 // needs density tiles in handle work memory), equal to esmf_fock_build within
 // that precision's tolerance.  Its FP64 J/K accumulators (the contraction

@@ -116,7 +116,7 @@ def ncu_traffic(kernel, precision, workload="stored_n200_m16"):
 
 # ------------------------------------------------------------------ ours
 DTYPES = {"fp64": "f64", "fp32": "f32", "fp16x2": "f16x2+f32acc", "bf16x2": "bf16x2+f32acc",
-          "f32x2": "f32x2 (double-FP32 hi+lo, error-free products)"}
+          "f32x2": "f32x2 (FP64 integrals as double-FP32 hi+lo)"}
 ELEM_BYTES = {"fp64": 8, "fp32": 4, "fp16x2": 4, "bf16x2": 4, "f32x2": 8}
 
 

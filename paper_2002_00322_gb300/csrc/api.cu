@@ -1336,7 +1336,7 @@ int build_df(esmf_fock_t *h, int m, const double *D, double *J, double *K, doubl
     if (h->dfTiles) {
         sp.n = h->n; sp.naux = h->naux; sp.m = m; sp.group = h->df_group; sp.num_sms = h->num_sms;
         sp.B = (const double *)h->dfB; sp.eB = h->dfeB; sp.nB = h->dfeB + h->n; sp.Btiles = h->dfTiles; sp.D = D;
-        sp.eD = h->dfeD; sp.ED = h->dfED; sp.top = h->dfED + h->df_m; sp.Dtiles = h->dfDtl; sp.Ytiles = h->dfYt; sp.S = (unsigned long long *)h->dfS;
+        sp.eD = h->dfeD; sp.ED = h->dfED; sp.top = h->dfED + m; sp.Dtiles = h->dfDtl; sp.Ytiles = h->dfYt; sp.S = (unsigned long long *)h->dfS;
         sp.K = (double *)h->dfKt; sp.error = h->err_dev;
     }
     DfBuild a;

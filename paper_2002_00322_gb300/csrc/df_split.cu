@@ -34,7 +34,7 @@
 // and Y is rounded to 2^-62 of its bound, which all columns share.
 //
 // Digits serve densities whose largest element lies in [2^-500, 2^500), where
-// the squares behind the bound on Y stay in FP64's range; k_df_plain takes the
+// the squares behind the bound on Y stay in FP64's range; plain_row takes the
 // others (and those with infinities or NaN) in FP64 arithmetic.  The factor's
 // elements are at most 2^250 (the handle keeps to cuBLAS otherwise).
 //
@@ -169,7 +169,7 @@ __global__ void k_df_btiles(const double *B, int naux, int n, int npb, int nkb, 
 // per density the exponent above max_s |D_k[:, s]|_2 in ED[k] (any smaller value
 // at launch; the column of the largest element has a norm in range and bounds the
 // columns whose squares underflow) and the exponent field of its largest element
-// in top[k] (0 at launch; subnormal elements count as 1).
+// in top[k] (below 0 at launch; subnormal elements count as 1).
 __global__ void k_df_dcols(const double *D, int n, int ldD, int16_t *eD, int *ED, int *top) {
     const int k = blockIdx.y, s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= ldD) return;
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_df_gemm(const __grid_constant
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             // right shift: nB > eB and ED > eD make it 10 at least (rows beyond n and
-                            // densities that k_df_plain takes get zeros)
+                            // densities that plain_row takes get zeros)
                             const int r = yp - ap - ed[g * 32 + i] + 70 - BITS;
                             const __int128 S = ((__int128)SH[g][i] << 36) + SL[g][i];
                             X[i] = r > 100 || r < 1 ? 0 : (long long)((S + ((__int128)1 << (r - 1))) >> r);
@@ -452,55 +452,51 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_df_gemm(const __grid_constant
     }
 }
 
-// K of a group's densities from their integer sums (each range adds less than
-// 2^36 to SL, and 2^18 blocks, more than the device has room for, 2^59 to SH)
-__global__ void k_df_kout(const __grid_constant__ DfGemm G, double *K) {
-    const int p = blockIdx.x, k = G.k0 + blockIdx.y;
-    if (beyond_digits(G.top[k])) return;
-    const unsigned long long *row = G.S + ((int64_t)blockIdx.y * G.n + p) * G.n;
-    const int e = G.nB[p] + G.ED[k] - 70;
-    for (int q = threadIdx.x; q < G.n; q += blockDim.x) {
-        const unsigned long long lo = row[q + (int64_t)G.kc * G.n * G.n];
-        const long long hi = (long long)(row[q] + (lo >> 36));
-        K[((int64_t)k * G.n + p) * G.n + q] = scalbn(fma((double)hi, 0x1p36, (double)(lo & SL_MASK)), e + G.eB[q]);
+// Row p of K of a density beyond the digits' range, in FP64 arithmetic:
+// y[s] = sum_r B[P][p][r] D[r][s] for a piece of s at a time, then K[p][q] += sum_s
+// y[s] B[P][s][q] (B is symmetric; both sums read whole rows).  200 functions, 700
+// auxiliaries: 41 ms a density (the two cuBLAS products took 27 ms).
+__device__ void plain_row(const double *B, const double *Dk, int n, int naux, int p, double *Kp) {
+    constexpr int PIECE = 1024;
+    __shared__ double y[PIECE];
+    for (int q = threadIdx.x; q < n; q += blockDim.x) Kp[q] = 0.0;
+    for (int P = 0; P < naux; ++P) {
+        const double *BP = B + (int64_t)P * n * n, *bp = BP + (int64_t)p * n;
+        for (int s0 = 0; s0 < n; s0 += PIECE) {
+            const int len = min(PIECE, n - s0);
+            __syncthreads();
+            for (int s = threadIdx.x; s < len; s += blockDim.x) {
+                double a = 0.0;
+                for (int r = 0; r < n; ++r) a = fma(bp[r], Dk[(int64_t)r * n + s0 + s], a);
+                y[s] = a;
+            }
+            __syncthreads();
+            for (int q = threadIdx.x; q < n; q += blockDim.x) {
+                double a = Kp[q];
+                for (int s = 0; s < len; ++s) a = fma(y[s], BP[(int64_t)(s0 + s) * n + q], a);
+                Kp[q] = a;
+            }
+        }
     }
 }
 
-// K of the densities beyond the digits' range, in FP64 arithmetic: a block forms
-// whole rows p, y[s] = sum_r B[P][p][r] D[r][s] for a piece of s at a time, then
-// K[p][q] += sum_s y[s] B[P][s][q] (B is symmetric; both sums read whole rows).
-// Others return at once.  200 functions, 700 auxiliaries: 34 ms a density (the
-// two cuBLAS products took 27 ms), FP64-bound.
-__global__ void __launch_bounds__(256) k_df_plain(const double *B, const double *D, int n, int naux, int m,
-                                                  const int *top, double *K) {
-    constexpr int PIECE = 1024;
-    __shared__ double y[PIECE];
-    const int64_t nn = (int64_t)n * n;
-    for (int k = 0; k < m; ++k) {
-        if (!beyond_digits(top[k])) continue;
-        const double *Dk = D + k * nn;
-        for (int p = blockIdx.x; p < n; p += gridDim.x) {
-            double *Kp = K + k * nn + (int64_t)p * n;
-            for (int q = threadIdx.x; q < n; q += blockDim.x) Kp[q] = 0.0;
-            for (int P = 0; P < naux; ++P) {
-                const double *BP = B + P * nn, *bp = BP + (int64_t)p * n;
-                for (int s0 = 0; s0 < n; s0 += PIECE) {
-                    const int len = min(PIECE, n - s0);
-                    __syncthreads();
-                    for (int s = threadIdx.x; s < len; s += blockDim.x) {
-                        double a = 0.0;
-                        for (int r = 0; r < n; ++r) a = fma(bp[r], Dk[(int64_t)r * n + s0 + s], a);
-                        y[s] = a;
-                    }
-                    __syncthreads();
-                    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-                        double a = Kp[q];
-                        for (int s = 0; s < len; ++s) a = fma(y[s], BP[(int64_t)(s0 + s) * n + q], a);
-                        Kp[q] = a;
-                    }
-                }
-            }
-        }
+// K of a group's densities, one block per row: from their integer sums (each range
+// adds less than 2^36 to SL, and 2^18 blocks, more than the device has room for,
+// 2^59 to SH), or by plain_row.
+__global__ void __launch_bounds__(256) k_df_kout(const __grid_constant__ DfGemm G, const double *B, const double *D, double *K) {
+    const int p = blockIdx.x, k = G.k0 + blockIdx.y;
+    const int64_t nn = (int64_t)G.n * G.n;
+    double *Kp = K + k * nn + (int64_t)p * G.n;
+    if (G.top[k] > 0 && beyond_digits(G.top[k])) {
+        plain_row(B, D + k * nn, G.n, G.naux, p, Kp);
+        return;
+    }
+    const unsigned long long *row = G.S + blockIdx.y * nn + (int64_t)p * G.n;
+    const int e = G.nB[p] + G.ED[k] - 70;
+    for (int q = threadIdx.x; q < G.n; q += blockDim.x) {
+        const unsigned long long lo = row[q + G.kc * nn];
+        const long long hi = (long long)(row[q] + (lo >> 36));
+        Kp[q] = scalbn(fma((double)hi, 0x1p36, (double)(lo & SL_MASK)), e + G.eB[q]);
     }
 }
 
@@ -571,8 +567,7 @@ int launch_df_split_factor(const double *B, int naux, int n, const int16_t *eB, 
 
 int launch_df_split_exchange(const DfSplit &a, cudaStream_t s) {
     const int n = a.n, npb = row_blocks(n), nkb = sum_blocks(n), ldD = nkb * 64;
-    CKS(cudaMemsetAsync(a.top, 0, sizeof(int) * a.m, s));
-    CKS(cudaMemsetAsync(a.ED, 0x80, sizeof(int) * a.m, s));
+    CKS(cudaMemsetAsync(a.ED, 0x80, sizeof(int) * 2 * a.m, s));       // top follows
     k_df_dcols<<<dim3((ldD + 63) / 64, a.m), 64, 0, s>>>(a.D, n, ldD, a.eD, a.ED, a.top);
     CKS(cudaGetLastError());
     k_df_dtiles<<<grid_for((int64_t)a.m * npb * nkb * 1024), 256, 0, s>>>(a.D, n, a.m, npb, nkb, ldD, a.eD, a.Dtiles);
@@ -593,11 +588,9 @@ int launch_df_split_exchange(const DfSplit &a, cudaStream_t s) {
         CKS(cudaMemsetAsync(a.S, 0, df_split_sum_bytes(n, g.kc), s));
         rc = df_gemm<true>(g, a.num_sms, s);
         if (rc != ESMF_OK) return rc;
-        k_df_kout<<<dim3(n, g.kc), n <= 128 ? 128 : 256, 0, s>>>(g, a.K);
+        k_df_kout<<<dim3(n, g.kc), n <= 128 ? 128 : 256, 0, s>>>(g, a.B, a.D, a.K);
         CKS(cudaGetLastError());
     }
-    k_df_plain<<<n < 4 * a.num_sms ? n : 4 * a.num_sms, 256, 0, s>>>(a.B, a.D, n, a.naux, a.m, a.top, a.K);
-    CKS(cudaGetLastError());
     return ESMF_OK;
 }
 

@@ -185,7 +185,7 @@ struct DfSplit {
     const unsigned char *Btiles;
     const double *D;
     int16_t *eD;                                 // work: column exponents, m x 64 ceil(n / 64)
-    int *ED, *top;                               // work: per density
+    int *ED, *top;                               // work: per density, top = ED + m
     unsigned char *Dtiles, *Ytiles;              // work: m matrices, group * naux matrices
     unsigned long long *S;                       // work: df_split_sum_bytes(n, group)
     double *K;                                   // m x n x n
